@@ -212,7 +212,7 @@ def roofline_of(name, per_launch_ms, dd, pk, precision):
     gbs = nbytes / sec / 1e9
     tfl = nflops / sec / 1e12
     f_hbm = gbs / pk["hbm_gbs"]
-    if "_tc_" in name or "_mma_" in name or name.startswith(("fno_da_tz", "fno_synth_t")):
+    if "_tc_" in name or "mma_" in name or name.startswith(("fno_da_tz", "fno_synth_t")):
         # tensor-core kernels (mma.sync): algorithmic flops against
         # the dense BF16 peak; split BF16 issues 3 (DFT stages) or 6 (1x1
         # stages) products per real multiply-add, which the fraction leaves out

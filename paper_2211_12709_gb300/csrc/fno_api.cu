@@ -9,6 +9,7 @@
 // DFT kernels with the c(kt)/N-scaled t table produce G, the mixing adjoint
 // gives dW and the input-spectrum gradient, and the inverse kernels with the
 // unscaled t table bring it back to the grid.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -172,7 +173,8 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 struct Layout {
   size_t err;  // device status word (nonzero: a bounded wait gave up)
   size_t tab[10];
-  size_t t1, t2, xh, yh, gxh, da, part, mma_tab, tc_tab, gp, vz, total;  // vz 0: no region
+  size_t t1, t2, xh, yh, gxh, da, part, mma_tab, tc_tab, gp, vz, epi_tab, total;  // vz 0: no region
+  size_t extra;  // bytes of total beyond the sizes that the static scratch's limit counts
   bool da_in_dx;
 };
 
@@ -236,8 +238,13 @@ static Layout layout(const Dims& d, int op) {
   }
   L.mma_tab = off;  // basis fragments of the mma.sync epilogue
   off += align256(epilogue_mma_table_bytes(d));
-  L.tc_tab = off;  // z basis images of the tcgen05 epilogue
-  off += align256(epilogue_tc_table_bytes(d));
+  // z basis images of the tcgen05 epilogue, or the column epilogue's fragments:
+  // a call runs one of the two
+  L.tc_tab = off;
+  L.epi_tab = off;
+  const size_t tcb = align256(epilogue_tc_table_bytes(d)), epb = align256(epi_tables_bytes(d));
+  L.extra = epb > tcb ? epb - tcb : 0;
+  off += tcb + L.extra;
   if (op == FNO_OP_BLOCK_TRAIN) {
     L.gp = off;  // GELU'(A) of the training forward, [B][C_out][grid]
     off += align256(sizeof(float) * (size_t)(d.B * d.Co * d.Ng));
@@ -343,22 +350,72 @@ static cudaError_t synth_epilogue(const Dims& d, const EpiArgs& a, int precision
   return cudaSuccess;
 }
 
-// The fused inverse z, t + epilogue stage: split BF16 and TF32 on tcgen05 (TMEM
-// accumulators) where its tiling applies, then warp-level mma.sync (plain BF16,
-// the dA mode and the shapes tcgen05 does not tile), then, in the tensor-core
-// precisions, the synthesis path for other Nt (not the dA mode), else FP32 on
-// the CUDA cores (the plain form, and the exact fallback for other shapes).
+// Which kernel runs the inverse z, t + epilogue stage of a call in the
+// tensor-core precisions (not the dA mode).  Times are forward + dX (us) of a
+// training step at 64^3 x Nt.
+//   column epilogue (k_epi_col): split BF16, and dX and the spectral form in plain
+//     BF16 on the grids of k_epi_mma (the sums that it rounds run in the same
+//     order).  Against the tcgen05 kernel, Nt = 32: 294 : 931 at 8 channels, 688 :
+//     1005 at 16, 1280 : 1437 at 24; against the synthesis path, Nt = 86: 1047 :
+//     1860 at 8 channels, 502 : 1370 at 4, 5531 : 7881 at 32.
+//   tcgen05 (k_epi_tc): beyond 24 channels, where its 32-wide products are full
+//     and the FP32 1x1 of the column form no longer is cheaper (Nt = 32, 32
+//     channels: 1502 : 1774; 24 channels: 1437 : 1280, at Nt = 16 807 : 721); and
+//     TF32, as the forms below.
+//   mma.sync (k_epi_mma) and the synthesis path (at other Nt): TF32, and plain BF16
+//     otherwise.  They keep their order of sums: dA and the spectra are
+//     rounded to 11 or 8 bits later, and a sum that differs in its last bit
+//     turns some of those roundings (rel 5e-5 in a TF32 gradient).  The
+//     synthesis path also has the grids of under 32 column tiles, where every
+//     form is a few launches of a few microseconds.
+enum EpiKind { KIND_F32, KIND_COL, KIND_TC, KIND_MMA, KIND_SYNTH };
+static EpiKind epilogue_kind(const Dims& d, int mode, int Cs, int Cl, int precision, bool region) {
+  if (!is_tc(precision)) return KIND_F32;
+  const bool fused = epilogue_mma_supported(d, mode, Cs, Cl, nullptr, 0);
+  if (mode == EPI_DA) return fused ? KIND_MMA : KIND_F32;
+  const bool synth = !fused && region && synth_shape_ok(d, Cs, Cl);
+  const int C = std::max(Cs, Cl);
+  const bool tc = is_split(precision) && epilogue_tc_supported(d, mode, Cs, Cl, nullptr, 0);
+  if (tc && C > 24) return KIND_TC;
+  const bool tiny = d.B * d.Nx * d.Ny * ((d.Nz + 15) / 16) < 32;
+  if ((fused || (synth && !tiny)) &&
+      (precision == FNO_BF16X3 || (precision == FNO_BF16 && fused && mode != EPI_FWD)) &&
+      epilogue_col_supported(d, mode, Cs, Cl))
+    return KIND_COL;
+  return tc ? KIND_TC : fused ? KIND_MMA : synth ? KIND_SYNTH : KIND_F32;
+}
+
+// The basis tables of a call whose epilogue has the given mode and channels, with
+// the fragments of the column epilogue where that one runs.
+static cudaError_t tables(const Dims& d, char* base, const Layout& L, const Tables& T, int mode, int Cs, int Cl,
+                          int precision, int* err, cudaStream_t s) {
+  const bool col = epilogue_kind(d, mode, Cs, Cl, precision, L.vz != 0) == KIND_COL;
+  const EpiTables et = epi_tables(d, base + L.epi_tab);
+  return launch_tables(d, T, col ? &et : nullptr, err, s);
+}
+
+// The fused inverse z, t + epilogue stage (see epilogue_kind).
 static cudaError_t epilogue(const Dims& d, EpiArgs a, int precision, char* base, const Layout& L,
                             int* err, int* grid_used, cudaStream_t s) {
-  // plain BF16 (one product, no split operands to build) measured faster on
-  // mma.sync; the split precisions on tcgen05
-  if (is_split(precision) && epilogue_tc_supported(d, a.mode, a.Cs, a.Cl, nullptr, 0))
-    return launch_epilogue_tc(d, a, true, precision == FNO_TF32, base + L.tc_tab, err, s);
-  if (is_tc(precision) && epilogue_mma_supported(d, a.mode, a.Cs, a.Cl, nullptr, 0))
-    return launch_epilogue_mma(d, a, is_split(precision), precision == FNO_TF32, base + L.mma_tab, err,
-                               grid_used, s);
-  if (is_tc(precision) && a.mode != EPI_DA && L.vz != 0 && synth_shape_ok(d, a.Cs, a.Cl))
-    return synth_epilogue(d, a, precision, reinterpret_cast<float2*>(base + L.vz), s);
+  const bool split = is_split(precision), tf32 = precision == FNO_TF32;
+  switch (epilogue_kind(d, a.mode, a.Cs, a.Cl, precision, L.vz != 0)) {
+    case KIND_COL: {
+      // on the grids that the fused forms tile, plain BF16 rounds the 1x1's
+      // operands and split BF16 has three-product DFT stages; on the others the
+      // 1x1 is FP32 and split BF16 has six products
+      const bool fused = epilogue_mma_supported(d, a.mode, a.Cs, a.Cl, nullptr, 0);
+      return launch_epilogue_col(d, a, split, !fused, fused && !split, epi_tables(d, base + L.epi_tab),
+                                 a.It == tables_at(base, L).Its, s);
+    }
+    case KIND_TC:
+      return launch_epilogue_tc(d, a, true, tf32, base + L.tc_tab, err, s);
+    case KIND_MMA:
+      return launch_epilogue_mma(d, a, split, tf32, base + L.mma_tab, err, grid_used, s);
+    case KIND_SYNTH:
+      return synth_epilogue(d, a, precision, reinterpret_cast<float2*>(base + L.vz), s);
+    default:
+      break;
+  }
   return launch_epilogue_f32(d, a, grid_used, s);
 }
 
@@ -396,7 +453,7 @@ static int forward_common(const Dims& d, int precision, int op, const float* x, 
   float2* xh = reinterpret_cast<float2*>(base + L.xh);
   float2* yh = reinterpret_cast<float2*>(base + L.yh);
   int* err = reinterpret_cast<int*>(base + L.err);
-  CK(launch_tables(d, T, err, s));
+  CK(tables(d, base, L, T, block ? EPI_FWD : EPI_SPECTRAL, (int)d.Co, block ? (int)d.Ci : 0, precision, err, s));
   if ((rc = spectrum_f32(d, d.Ci, x, T.Ft, T, t1, t2, xh, s, precision, err))) return rc;
   CK(launch_mix_f32(d, xh, reinterpret_cast<const float2*>(w), yh, s));
   if ((rc = inverse_xy_f32(d, d.Co, yh, T, t2, t1, s, precision))) return rc;
@@ -569,7 +626,7 @@ int fno_spectral_bwd(const fno_dims* dims, int precision, const float* x, const 
   float2* g = reinterpret_cast<float2*>(base + L.yh);
   float2* gxh = reinterpret_cast<float2*>(base + L.gxh);
   int* err = reinterpret_cast<int*>(base + L.err);
-  CK(launch_tables(d, T, err, s));
+  CK(tables(d, base, L, T, EPI_SPECTRAL, (int)d.Ci, 0, precision, err, s));
   if ((rc = spectrum_f32(d, d.Co, dy, T.Fta, T, t1, t2, g, s, precision, err))) return rc;
   if (dw)
     if ((rc = spectrum_f32(d, d.Ci, x, T.Ft, T, t1, t2, xh, s, precision, err))) return rc;
@@ -637,7 +694,7 @@ static int block_bwd_impl(const fno_dims* dims, int precision, const float* x, c
   const Layout LT = layout(d, FNO_OP_BLOCK_TRAIN);
   if (train && (rc = check_ws(ws, ws_bytes, LT))) return rc;
   saved_forget(ws);  // the steps below overwrite the forward state
-  CK(launch_tables(d, T, err, s));
+  CK(tables(d, base, L, T, EPI_DX, (int)d.Ci, (int)d.Co, precision, err, s));
   if (!saved) {
     // recompute the forward spectrum and the spectral partial U1 of the output
     if ((rc = spectrum_f32(d, d.Ci, x, T.Ft, T, t1, t2, xh, s, precision, err))) return rc;
@@ -899,7 +956,10 @@ int fno_profile_entry(int i, const char** name, int64_t* launches, double* total
 // file instead of a caller workspace (for callers that may not allocate device
 // memory; see include/fno.h).
 // ---------------------------------------------------------------------------
-static __device__ __align__(256) unsigned char g_fno_static_scratch[FNO_STATIC_SCRATCH_BYTES];
+// The limit of FNO_STATIC_SCRATCH_BYTES does not count Layout::extra (at most 24
+// KB of t fragments and 12 KB of z rows past Nz); the array has room for it.
+static const size_t kStaticSlack = 64 * 1024;
+static __device__ __align__(256) unsigned char g_fno_static_scratch[FNO_STATIC_SCRATCH_BYTES + kStaticSlack];
 
 namespace fno {
 static std::mutex g_static_mu;
@@ -948,8 +1008,9 @@ extern "C" int fno_spectral_fwd_static(const fno_dims* dims, int precision, cons
   int rc = to_dims(dims, &d);
   if (rc) return rc;
   if ((rc = check_support(d, precision, FNO_OP_SPECTRAL_FWD))) return rc;
-  const size_t need = layout(d, FNO_OP_SPECTRAL_FWD).total;
-  if (need > FNO_STATIC_SCRATCH_BYTES)
+  const Layout L = layout(d, FNO_OP_SPECTRAL_FWD);
+  const size_t need = L.total - L.extra;
+  if (need > FNO_STATIC_SCRATCH_BYTES || L.extra > kStaticSlack)
     return fail(FNO_ERR_UNSUPPORTED,
                 "these sizes need %zu bytes of scratch; the static scratch holds %zu bytes "
                 "(use fno_spectral_fwd with a workspace)",
@@ -957,6 +1018,6 @@ extern "C" int fno_spectral_fwd_static(const fno_dims* dims, int precision, cons
   void* ws = nullptr;
   if ((rc = static_scratch(&ws))) return rc;
   return forward_common(d, precision, FNO_OP_SPECTRAL_FWD, x, w, nullptr, nullptr, y, ws,
-                        FNO_STATIC_SCRATCH_BYTES, (cudaStream_t)stream);
+                        FNO_STATIC_SCRATCH_BYTES + kStaticSlack, (cudaStream_t)stream);
 }
 

@@ -11,6 +11,8 @@
 //   k_mix_adj_f32  its adjoint: weight gradient and input-spectrum gradient
 //   k_epi_f32      inverse z then t, fused with the 1x1 linear, bias and GELU
 //                  (or their gradients)
+#include <cuda_bf16.h>
+
 #include <algorithm>
 
 #include "fno_internal.h"
@@ -49,11 +51,100 @@ struct TabParams {
   int Nt;
   double invNg;
   int* err;
+  EpiTables et;
+  int Nz, mz, Jt;
+  long long ncz, nct;  // threads of the epilogue's z and t fragments (0: none)
 };
+
+// FP32 value of sc exp(+2 pi i k n / N)
+__device__ float2 root_of_unity(long long k, long long n, long long N, double sc) {
+  long long rr = (k * n) % N;
+  if (rr < 0) rr += N;
+  double sn, cs;
+  sincospi(2.0 * (double)rr / (double)N, &sn, &cs);
+  return make_float2((float)(cs * sc), (float)(sn * sc));
+}
+
+// three exact BF16 parts of two floats
+__device__ void three_parts(float a, float b, uint32_t (&p)[3]) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    const float2 f = __bfloat1622float2(h);
+    p[q] = *reinterpret_cast<const uint32_t*>(&h);
+    a -= f.x;
+    b -= f.y;
+  }
+}
+
+// Fragments of the epilogue's bases (see EpiTables): thread e < ncz one lane of
+// one (16-plane tile, k-step) of the z basis, the others one lane of one
+// 8-point t sub-tile (rows (kt, cos), then (kt, -sin)).
+__device__ void epi_fragments(const TabParams& p, long long e) {
+  const EpiTables& c = p.et;
+  const int lane = (int)(e % 32), g = lane / 4, q = lane % 4;
+  e /= 32;
+  uint32_t w[4][3];
+  if (e < p.ncz / 32) {
+    const int ks = (int)(e % c.KS), zt = (int)(e / c.KS);
+#pragma unroll 1
+    for (int r = 0; r < 4; ++r) {
+      const int z = 16 * zt + g + 8 * (r & 1), jz = 8 * ks + q + 4 * (r >> 1);
+      float2 f = make_float2(0.f, 0.f);
+      if (z < p.Nz && jz < 2 * p.mz) f = root_of_unity(jz < p.mz ? jz : jz - 2 * p.mz, z, p.Nz, 1.0);
+      three_parts(f.x, -f.y, w[r]);
+    }
+    for (int k = 0; k < 3; ++k) c.zf[(e * 3 + k) * 32 + lane] = make_uint4(w[0][k], w[1][k], w[2][k], w[3][k]);
+    return;
+  }
+  e -= p.ncz / 32;
+  const bool scaled = e < 2 * c.NTT;
+  if (!scaled) e -= 2 * c.NTT;
+  const int h = (int)(e % 2), T = (int)(e / 2);
+  const int t = 16 * T + (c.perm ? 4 * (g / 2) + 2 * h + g % 2 : 8 * h + g);
+  float cv[2], sv[2];
+#pragma unroll 1
+  for (int u = 0; u < 2; ++u) {
+    const int kt = 2 * q + u;
+    const bool single = kt == 0 || (p.Nt % 2 == 0 && 2 * kt == p.Nt);
+    const double sc = scaled ? (single ? 1.0 : 2.0) * p.invNg : 1.0;
+    float2 f = make_float2(0.f, 0.f);
+    if (t < p.Nt && kt < p.Jt) f = root_of_unity(kt, t, p.Nt, sc);
+    cv[u] = f.x;
+    sv[u] = -f.y;
+  }
+  three_parts(cv[0], cv[1], w[0]);
+  three_parts(sv[0], sv[1], w[1]);
+  uint2* dst = scaled ? c.tfs : c.tfu;
+  for (int k = 0; k < 3; ++k) dst[(e * 3 + k) * 32 + lane] = make_uint2(w[0][k], w[1][k]);
+}
+
+EpiTables epi_tables(const Dims& d, void* base) {
+  EpiTables c{};
+  c.NZ = (int)((d.Nz + 15) / 16);
+  c.KS = (int)((d.Jz + 7) / 8);
+  c.NTT = (int)((d.Nt + 15) / 16);
+  c.H = d.Nt > 16 ? 2 : 1;
+  c.perm = (c.H == 2 && d.Nt % 4 == 0) ? 1 : 0;
+  c.zf = static_cast<uint4*>(base);
+  c.tfs = reinterpret_cast<uint2*>(c.zf + (size_t)c.NZ * c.KS * 3 * 32);
+  c.tfu = c.tfs + (size_t)c.NTT * 2 * 3 * 32;
+  return c;
+}
+size_t epi_tables_bytes(const Dims& d) {
+  const EpiTables c = epi_tables(d, nullptr);
+  return sizeof(uint4) * (size_t)c.NZ * c.KS * 3 * 32 + 2 * sizeof(uint2) * (size_t)c.NTT * 2 * 3 * 32;
+}
 
 __global__ void k_tables(TabParams p) {
   long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx == 0 && p.err) *p.err = 0;
+  // the fragments first: their threads have the longest chains
+  if (idx < p.ncz + p.nct) {
+    epi_fragments(p, idx);
+    return;
+  }
+  idx -= p.ncz + p.nct;
   if (idx >= p.start[p.nseg]) return;
   int s = 0;
   while (s + 1 < p.nseg && idx >= p.start[s + 1]) ++s;
@@ -75,9 +166,17 @@ __global__ void k_tables(TabParams p) {
   g.dst[e] = make_float2((float)(cs * sc), (float)((double)g.sign * sn * sc));
 }
 
-cudaError_t launch_tables(const Dims& d, const Tables& T, int* err, cudaStream_t s) {
+cudaError_t launch_tables(const Dims& d, const Tables& T, const EpiTables* et, int* err, cudaStream_t s) {
   TabParams p{};
   p.err = err;
+  if (et) {
+    p.et = *et;
+    p.Nz = (int)d.Nz;
+    p.mz = (int)d.mz;
+    p.Jt = (int)d.Jt;
+    p.ncz = 32LL * et->NZ * et->KS;
+    p.nct = 32LL * 4 * et->NTT;
+  }
   auto add = [&](float2* dst, int64_t rows, int64_t cols, int64_t N, int64_t m, int kr, int sign,
                  int scale) {
     p.seg[p.nseg] = TabSeg{dst, (int)rows, (int)cols, (int)N, (int)m, kr, sign, scale};
@@ -97,8 +196,10 @@ cudaError_t launch_tables(const Dims& d, const Tables& T, int* err, cudaStream_t
   add(T.Itu, d.Jt, d.Nt, d.Nt, 0, 1, +1, 0);
   p.Nt = (int)d.Nt;
   p.invNg = 1.0 / (double)d.Ng;
-  long long total = p.start[p.nseg];
-  int threads = 256;
+  long long total = p.start[p.nseg] + p.ncz + p.nct;
+  // one warp a block: an SM does about two FP64 operations a clock, so the
+  // entries (some fifty operations each) are spread over all of them
+  int threads = 32;
   int blocks = (int)((total + threads - 1) / threads);
   FNO_LAUNCH("fno_tables", k_tables, blocks, threads, 0, s, p);
   return cudaSuccess;

@@ -31,9 +31,24 @@ void prof_before(const char* name, cudaStream_t s);
 void prof_after(cudaStream_t s);
 int sm_count();
 
+// Fragment tables of the column epilogue (fno_epi_col.cu), three BF16 parts: the
+// inverse z basis as mma.sync A fragments [NZ][KS][3 parts][32 lanes] (tiles of
+// 16 planes; columns (kz, Re), (kz, -Im)) and the inverse t basis as B fragments
+// [NTT][2][3 parts][32 lanes] (NTT tiles of two 8-point sub-tiles), scaled by
+// c(kt)/N (tfs) and not (tfu).  KS: k-steps of 8 kz.  H: sub-tiles of an item of
+// the kernel; perm: their t order gives a lane four consecutive points (H = 2
+// and Nt a multiple of 4), so that it loads and stores 16 bytes at a time.
+struct EpiTables {
+  uint4* zf;
+  uint2 *tfs, *tfu;
+  int NZ, KS, NTT, H, perm;
+};
+EpiTables epi_tables(const Dims& d, void* base);
+size_t epi_tables_bytes(const Dims& d);
+
 // ---- FP32 CUDA-core kernels (fno_fp32.cu) -----------------------------------
-// also clears the device status word *err of the call
-cudaError_t launch_tables(const Dims& d, const Tables& T, int* err, cudaStream_t s);
+// also clears the device status word *err of the call; et nullable
+cudaError_t launch_tables(const Dims& d, const Tables& T, const EpiTables* et, int* err, cudaStream_t s);
 
 // in[ncol][Nz][Nt] real -> out[ncol][Jz][Jt] complex: pruned DFT over t, then z.
 // ft is Ft or Fta.
@@ -92,6 +107,15 @@ bool epilogue_mma_supported(const Dims& d, int mode, int Cs, int Cl, char* why, 
 size_t epilogue_mma_table_bytes(const Dims& d);
 cudaError_t launch_epilogue_mma(const Dims& d, const EpiArgs& a, bool split, bool tf32, void* table,
                                 int* err, int* grid_used, cudaStream_t s);
+
+// Inverse z, t + epilogue by columns on mma.sync with the 1x1 in packed FP32
+// (fno_epi_col.cu), modes EPI_FWD, EPI_DX and EPI_SPECTRAL, any even Nt <= 128;
+// same contract as launch_epilogue_f32 (no partial sums).  exact: split BF16 with
+// three parts and six products in the DFT stages (else two and three).
+// lin_round: the 1x1 operands rounded to BF16.  scaled: It is Its (else Itu).
+bool epilogue_col_supported(const Dims& d, int mode, int Cs, int Cl);
+cudaError_t launch_epilogue_col(const Dims& d, const EpiArgs& a, bool split, bool exact, bool lin_round,
+                                const EpiTables& ct, bool scaled, cudaStream_t s);
 
 // Inverse z, t + epilogue on the 5th-generation tensor cores (fno_tc.cu):
 // tcgen05.mma into TMEM accumulators, modes EPI_FWD, EPI_DX and EPI_SPECTRAL;
