@@ -182,6 +182,11 @@ cudaError_t launch_fwd_tz_mma(const float* in, float2* out, int64_t ncol, const 
                               const float2* ft, const float2* fz, bool split, bool tf32, int* err,
                               cudaStream_t s);
 
+// The same with the columns loaded straight into registers (fno_tz_reg.cu).
+bool fwd_tz_reg_supported(const Dims& d, bool split);
+cudaError_t launch_fwd_tz_reg(const float* in, float2* out, int64_t ncol, const Dims& d, const float2* ft,
+                              const float2* fz, bool split, bool tf32, cudaStream_t s);
+
 // The dA pass of a block backward after a training forward fused with the
 // forward pruned t, z DFT of dA (fno_da_tz.cu, mma.sync): writes da, the
 // spectrum t1 = [B Co Nx Ny][Jz][Jt] (ft = Fta) and at most max_rows partial

@@ -1802,6 +1802,7 @@ cudaError_t launch_fwd_tz_mma(const float* in, float2* out, int64_t ncol, const 
                               const float2* ft, const float2* fz, bool split, bool tf32, int* err,
                               cudaStream_t s) {
   if (ncol <= 0) return cudaSuccess;
+  if (fwd_tz_reg_supported(d, split || tf32)) return launch_fwd_tz_reg(in, out, ncol, d, ft, fz, split, tf32, s);
   TzM k{};
   size_t smem = 0;
   if (!tz_mma_plan(d, k, smem)) return cudaErrorInvalidValue;
