@@ -390,17 +390,25 @@ cudaError_t launch_line_f32(const float2* in, float2* out, int64_t outer, int ni
 //   forward  yh[b][o][j]  = sum_i xh[b][i][j] w[i][o][j]
 //   adjoint  gxh[b][i][j] = sum_o conj(w[i][o][j]) g[b][o][j]
 //            dw[i][o][j]  = sum_b conj(xh[b][i][j]) g[b][o][j]
-// A CTA owns a tile of kMixJ consecutive modes.  It stages the tile's spectra
-// for a chunk of BC batch entries in shared memory (rows of kMixJ complex
-// values: 128-byte coalesced loads), then each thread keeps one mode j of the
-// tile (lane % kMixJ) and walks the output channels of its group (tid / kMixJ,
-// stride kMixG), reading the weights straight from HBM in coalesced 128-byte
-// rows.  W, dW and the outputs cross HBM once per batch chunk (once when
-// B <= BC), and every sum runs in a fixed order.
+// A CTA owns a tile of kMixJ consecutive modes and has one group of kMixJ
+// threads per channel (output channels forward, input channels in the adjoint;
+// at most kMixG groups, which then take several in turn).  It stages the tile's
+// spectra for a chunk of BC batch entries in shared memory (rows of kMixJ
+// complex values: 128-byte coalesced loads), then each thread walks the summed
+// channel with kMixU weights in flight at a time, read straight from HBM in
+// coalesced 128-byte rows; the first ones are under way before the staging.  W,
+// dW and the outputs cross HBM once per batch chunk (once when B <= BC), and
+// every sum runs in a fixed order.
+// HBM bounds it (W, and dW in the adjoint).  With 16 fixed groups (20 channels:
+// two rounds, the second a quarter full) and 4 or 8 weights in flight the
+// forward and its adjoint took 59 and 57 us at 24576 modes, B = 2, width 20 (W 79
+// MB), here 27 and 42; 72 and 107, here 53 and 94 at 73728 modes, B = 1; 263 and
+// 361, here 207 and 354 at 110592 modes, B = 2, width 32.  20 weights in flight
+// measured slower (registers), 5 about as fast.
 // ---------------------------------------------------------------------------
-constexpr int kMixJ = 16;                   // modes per tile
-constexpr int kMixThreads = 256;
-constexpr int kMixG = kMixThreads / kMixJ;  // channel groups per tile
+constexpr int kMixJ = 16;  // modes per tile
+constexpr int kMixG = 32;  // most channel groups of a CTA
+constexpr int kMixU = 10;  // weights in flight per thread
 
 __device__ __forceinline__ void cmac(float2& acc, const float2 a, const float2 b) {
   acc.x = fmaf(a.x, b.x, acc.x);
@@ -419,39 +427,53 @@ __device__ __forceinline__ void cmac_conj(float2& acc, const float2 a, const flo
 // stage src[b0 + q][c][j0 .. j0 + kMixJ) for q < nb, c < C into dst[q][c][kMixJ]
 __device__ __forceinline__ void mix_stage(float2* dst, const float2* __restrict__ src, int b0,
                                           int nb, int BC, int C, long long Mk, long long j0) {
-  for (int e = threadIdx.x; e < BC * C * kMixJ; e += kMixThreads) {
+  for (int e = threadIdx.x; e < BC * C * kMixJ; e += blockDim.x) {
     const int jl = e % kMixJ, c = (e / kMixJ) % C, q = e / (kMixJ * C);
     const long long j = j0 + jl;
     dst[e] = (q < nb && j < Mk) ? src[((long long)(b0 + q) * C + c) * Mk + j]
                                 : make_float2(0.f, 0.f);
   }
 }
+// weights u0 .. u0 + kMixU of a row of n, `step` apart
+__device__ __forceinline__ void mix_load(float2 (&wv)[kMixU], const float2* __restrict__ wp, long long step,
+                                         int u0, int n, bool in) {
+#pragma unroll
+  for (int u = 0; u < kMixU; ++u)
+    wv[u] = (in && u0 + u < n) ? __ldg(wp + (u0 + u) * step) : make_float2(0.f, 0.f);
+}
 
 template <int BC>
-__global__ void __launch_bounds__(kMixThreads)
+__global__ void __launch_bounds__(kMixJ * kMixG, 2)
     k_mix_f32(const float2* __restrict__ xh, const float2* __restrict__ w, float2* __restrict__ yh,
               int B, int Ci, int Co, long long Mk) {
   extern __shared__ float2 mix_sm[];
   float2* xs = mix_sm;  // [BC][Ci][kMixJ]
-  const int jl = threadIdx.x % kMixJ, grp = threadIdx.x / kMixJ;
+  const int jl = threadIdx.x % kMixJ, grp = threadIdx.x / kMixJ, ngrp = blockDim.x / kMixJ;
   const long long j0 = (long long)blockIdx.x * kMixJ, j = j0 + jl;
   const bool inj = j < Mk;
+  const long long step = (long long)Co * Mk;
   for (int b0 = 0; b0 < B; b0 += BC) {
     const int nb = min(BC, B - b0);
+    float2 wv[kMixU];
+    mix_load(wv, w + (long long)grp * Mk + j, step, 0, Ci, inj);
     __syncthreads();
     mix_stage(xs, xh, b0, nb, BC, Ci, Mk, j0);
     __syncthreads();
     if (!inj) continue;
-    for (int o = grp; o < Co; o += kMixG) {
+    for (int o = grp; o < Co; o += ngrp) {
       float2 acc[BC];
 #pragma unroll
       for (int q = 0; q < BC; ++q) acc[q] = make_float2(0.f, 0.f);
       const float2* wp = w + (long long)o * Mk + j;
-#pragma unroll 4
-      for (int i = 0; i < Ci; ++i) {
-        const float2 wv = __ldg(wp + (long long)i * Co * Mk);
+      for (int i0 = 0; i0 < Ci; i0 += kMixU) {
+        if (i0 > 0 || o != grp) mix_load(wv, wp, step, i0, Ci, true);
 #pragma unroll
-        for (int q = 0; q < BC; ++q) cmac(acc[q], xs[(q * Ci + i) * kMixJ + jl], wv);
+        for (int u = 0; u < kMixU; ++u) {
+          if (i0 + u < Ci) {
+#pragma unroll
+            for (int q = 0; q < BC; ++q) cmac(acc[q], xs[(q * Ci + i0 + u) * kMixJ + jl], wv[u]);
+          }
+        }
       }
 #pragma unroll
       for (int q = 0; q < BC; ++q)
@@ -461,50 +483,58 @@ __global__ void __launch_bounds__(kMixThreads)
 }
 
 template <int BC>
-__global__ void __launch_bounds__(kMixThreads)
+__global__ void __launch_bounds__(kMixJ * kMixG, 2)
     k_mix_adj_f32(const float2* __restrict__ xh, const float2* __restrict__ w,
                   const float2* __restrict__ g, float2* __restrict__ dw, float2* __restrict__ gxh,
                   int B, int Ci, int Co, long long Mk) {
   extern __shared__ float2 mix_sm[];
   float2* xs = mix_sm;                   // [BC][Ci][kMixJ]
   float2* gs = mix_sm + BC * Ci * kMixJ; // [BC][Co][kMixJ]
-  const int jl = threadIdx.x % kMixJ, grp = threadIdx.x / kMixJ;
+  const int jl = threadIdx.x % kMixJ, grp = threadIdx.x / kMixJ, ngrp = blockDim.x / kMixJ;
   const long long j0 = (long long)blockIdx.x * kMixJ, j = j0 + jl;
   const bool inj = j < Mk;
   for (int b0 = 0; b0 < B; b0 += BC) {
     const int nb = min(BC, B - b0);
+    float2 wv[kMixU];
+    mix_load(wv, w + (long long)grp * Co * Mk + j, Mk, 0, Co, inj && gxh);
     __syncthreads();
     if (dw) mix_stage(xs, xh, b0, nb, BC, Ci, Mk, j0);
     mix_stage(gs, g, b0, nb, BC, Co, Mk, j0);
     __syncthreads();
     if (!inj) continue;
     if (gxh) {
-      for (int i = grp; i < Ci; i += kMixG) {
+      for (int i = grp; i < Ci; i += ngrp) {
         float2 ga[BC];
 #pragma unroll
         for (int q = 0; q < BC; ++q) ga[q] = make_float2(0.f, 0.f);
         const float2* wp = w + (long long)i * Co * Mk + j;
-#pragma unroll 8
-        for (int o = 0; o < Co; ++o) {
-          const float2 wv = __ldg(wp + (long long)o * Mk);
+        for (int o0 = 0; o0 < Co; o0 += kMixU) {
+          if (o0 > 0 || i != grp) mix_load(wv, wp, Mk, o0, Co, true);
 #pragma unroll
-          for (int q = 0; q < BC; ++q) cmac_conj(ga[q], wv, gs[(q * Co + o) * kMixJ + jl]);
+          for (int u = 0; u < kMixU; ++u) {
+            if (o0 + u < Co) {
+#pragma unroll
+              for (int q = 0; q < BC; ++q) cmac_conj(ga[q], wv[u], gs[(q * Co + o0 + u) * kMixJ + jl]);
+            }
+          }
         }
 #pragma unroll
         for (int q = 0; q < BC; ++q)
           if (q < nb) gxh[((long long)(b0 + q) * Ci + i) * Mk + j] = ga[q];
       }
     }
+    // dW after it: reads of W and writes of dW in one loop measured slower
     if (dw) {
-      for (int i = 0; i < Ci; ++i) {
+      for (int i = grp; i < Ci; i += ngrp) {
         float2 xv[BC];
 #pragma unroll
         for (int q = 0; q < BC; ++q) xv[q] = xs[(q * Ci + i) * kMixJ + jl];
-        for (int o = grp; o < Co; o += kMixG) {
+        float2* dp = dw + (long long)i * Co * Mk + j;
+#pragma unroll 4
+        for (int o = 0; o < Co; ++o, dp += Mk) {
           float2 da = make_float2(0.f, 0.f);
 #pragma unroll
           for (int q = 0; q < BC; ++q) cmac_conj(da, xv[q], gs[(q * Co + o) * kMixJ + jl]);
-          float2* dp = dw + ((long long)i * Co + o) * Mk + j;
           if (b0 == 0) {
             *dp = da;
           } else {
@@ -517,6 +547,11 @@ __global__ void __launch_bounds__(kMixThreads)
   }
 }
 
+// Input-channel groups of the adjoint: one each up to 24 channels, else two in
+// turn (32 channels, B = 2: 330 us in 16 groups, 371 in 32; 20 channels: 46 in 16,
+// 38 in 20).
+static int mix_adj_groups(int64_t Ci) { return (int)(Ci <= 24 ? Ci : (Ci + 1) / 2); }
+
 static int mix_bc(int64_t B) { return B <= 1 ? 1 : B <= 2 ? 2 : B <= 4 ? 4 : 8; }
 
 template <int BC>
@@ -528,7 +563,7 @@ static cudaError_t launch_mix_bc(const Dims& d, const float2* xh, const float2* 
     if (e != cudaSuccess) return e;
   }
   const unsigned grid = (unsigned)((d.Mk + kMixJ - 1) / kMixJ);
-  FNO_LAUNCH("fno_mix_f32", k_mix_f32<BC>, grid, kMixThreads, smem, s, xh, w, yh, (int)d.B,
+  FNO_LAUNCH("fno_mix_f32", k_mix_f32<BC>, grid, kMixJ * (int)std::min<int64_t>(kMixG, d.Co), smem, s, xh, w, yh, (int)d.B,
              (int)d.Ci, (int)d.Co, (long long)d.Mk);
   return cudaSuccess;
 }
@@ -542,7 +577,7 @@ static cudaError_t launch_mix_adj_bc(const Dims& d, const float2* xh, const floa
     if (e != cudaSuccess) return e;
   }
   const unsigned grid = (unsigned)((d.Mk + kMixJ - 1) / kMixJ);
-  FNO_LAUNCH("fno_mix_adjoint_f32", k_mix_adj_f32<BC>, grid, kMixThreads, smem, s, xh, w, g, dw,
+  FNO_LAUNCH("fno_mix_adjoint_f32", k_mix_adj_f32<BC>, grid, kMixJ * mix_adj_groups(d.Ci), smem, s, xh, w, g, dw,
              gxh, (int)d.B, (int)d.Ci, (int)d.Co, (long long)d.Mk);
   return cudaSuccess;
 }
