@@ -209,111 +209,297 @@ cudaError_t launch_tables(const Dims& d, const Tables& T, const EpiTables* et, i
 // Forward pruned DFT over t, then z, of each column [Nz][Nt] (real input):
 //   P[z][jt]  = sum_t x[z][t] ft[jt][t]
 //   T1[jz][jt] = sum_z fz[jz][z] P[z][jt]
-// One CTA walks columns (persistent); one thread per z row in the t stage and
-// per (jz, jt) output in the z stage.
+// One warp per column.  t stage: a lane owns one or two z rows and folds t and
+// Nt - t (the sum meets the cosines, the difference the sines), so a basis value
+// read once (16-byte broadcasts) serves two points of each row.  z stage: a lane
+// owns one jt and up to three |kz| and folds z and Nz - z likewise; the sums over
+// cosines and sines give +kz and -kz together.  Together a quarter of the
+// multiply-adds of the plain sums.
+// Rows of a multiple of four floats are read straight from global memory, 16
+// bytes per lane; other rows are copied to shared memory as they lie, 32 or 64 at
+// a time (an odd row stride has no bank conflicts, Nt % 4 = 2 two-way ones; whole
+// columns of 22 KB left eight warps on an SM and took 4.27 ms at 20 x 64^3 x 86).
+// Issue bounds it.  One thread per row and per output with one basis read per two
+// multiply-adds took 641 us at 2 x 20 x 64^3 x 16 and 132 us at 2 x 12 x 45 x 37
+// x 27 x 21; this form 314 and 66 (three CTAs of 80 registers on an SM; two: 314
+// and 82).
 // ---------------------------------------------------------------------------
 size_t fwd_tz_smem_bytes(const Dims& d) {
   return sizeof(float2) * (size_t)(d.Jt * d.Nt + d.Jz * (d.Nz + 1) + d.Nz * d.Jt);
 }
 
-template <bool VEC4>
-__global__ void __launch_bounds__(128)
+constexpr int kTzfP = 10;  // float2 stride of a row of P (8 used): 16-byte stores without conflicts
+
+// rows copied at a time (not V4)
+__host__ __device__ inline int tzf_rows_at_once(int Nz, int Nt) { return Nz > 32 && Nt <= 32 ? 64 : 32; }
+
+// shared memory of W warps: tables, then per warp P and (not V4) the rows
+static size_t tzf_smem(const Dims& d, bool v4, int W) {
+  const size_t tab = sizeof(float2) * ((size_t)((d.Jt + 7) / 8) * (d.Nt / 2 + 1) * 8 +
+                                       (((size_t)(d.Nz / 2 + 1) * (d.mz + 1) + 1) & ~(size_t)1));
+  const size_t col =
+      v4 ? 0 : sizeof(float) * (((size_t)std::min<int64_t>(d.Nz, tzf_rows_at_once((int)d.Nz, (int)d.Nt)) * d.Nt + 3) & ~(size_t)3);
+  return tab + (size_t)W * (sizeof(float2) * kTzfP * (size_t)d.Nz + col);
+}
+
+// t stage of rows z0 + lane + 32 r (r < R): P[z][0..7] of one group of eight jt.
+// F: [Nt / 2 + 1][8] (cos, -sin).
+template <bool V4, int R>
+__device__ __forceinline__ void tzf_rows(const float* __restrict__ src, float2* sP, const float2* F, int z0, int Nz,
+                                         int Nt, int lane) {
+  float ar[R][8], ai[R][8];
+  const float* row[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) row[r] = src + (long long)min(z0 + lane + 32 * r, Nz - 1) * Nt;
+  auto basis = [&](int t, float (&c)[8], float (&n)[8]) {
+    const float4* f = reinterpret_cast<const float4*>(F + t * 8);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 v = f[q];
+      c[2 * q] = v.x;
+      n[2 * q] = v.y;
+      c[2 * q + 1] = v.z;
+      n[2 * q + 1] = v.w;
+    }
+  };
+  // t and Nt - t
+  auto pair = [&](int t, const float (&u)[R], const float (&v)[R]) {
+    float c[8], n[8];
+    basis(t, c, n);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float s = u[r] + v[r], d = u[r] - v[r];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        ar[r][q] = fmaf(s, c[q], ar[r][q]);
+        ai[r][q] = fmaf(d, n[q], ai[r][q]);
+      }
+    }
+  };
+  // t = 0 and t = Nt / 2 stand alone; their sines are zero
+  auto single = [&](int t, const float (&u)[R]) {
+    float c[8], n[8];
+    basis(t, c, n);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) ar[r][q] = fmaf(u[r], c[q], ar[r][q]);
+  };
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) ar[r][q] = ai[r][q] = 0.f;
+  if (V4) {
+    // 16 bytes from the head and 16 from the tail of the rows at a time
+    float carry[R], u[R], v[R];
+    const int C = Nt / 8;
+#pragma unroll 1
+    for (int c = 0; c < C; ++c) {
+      float4 h[R], w[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        h[r] = __ldg(reinterpret_cast<const float4*>(row[r] + 4 * c));
+        w[r] = __ldg(reinterpret_cast<const float4*>(row[r] + Nt - 4 - 4 * c));
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) u[r] = h[r].x;
+      if (c == 0)
+        single(0, u);
+      else
+        pair(4 * c, u, carry);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        u[r] = h[r].y;
+        v[r] = w[r].w;
+      }
+      pair(4 * c + 1, u, v);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        u[r] = h[r].z;
+        v[r] = w[r].z;
+      }
+      pair(4 * c + 2, u, v);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        u[r] = h[r].w;
+        v[r] = w[r].y;
+        carry[r] = w[r].x;
+      }
+      pair(4 * c + 3, u, v);
+    }
+    if (Nt % 8 == 0) {
+      single(Nt / 2, carry);
+    } else {  // four values are left in the middle
+      float4 h[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) h[r] = __ldg(reinterpret_cast<const float4*>(row[r] + 4 * C));
+#pragma unroll
+      for (int r = 0; r < R; ++r) u[r] = h[r].x;
+      if (C == 0)
+        single(0, u);
+      else
+        pair(4 * C, u, carry);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        u[r] = h[r].y;
+        v[r] = h[r].w;
+      }
+      pair(4 * C + 1, u, v);
+#pragma unroll
+      for (int r = 0; r < R; ++r) u[r] = h[r].z;
+      single(Nt / 2, u);
+    }
+  } else {
+    float u[R], v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) u[r] = row[r][0];
+    single(0, u);
+#pragma unroll 2
+    for (int t = 1; 2 * t < Nt; ++t) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        u[r] = row[r][t];
+        v[r] = row[r][Nt - t];
+      }
+      pair(t, u, v);
+    }
+    if (Nt % 2 == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) u[r] = row[r][Nt / 2];
+      single(Nt / 2, u);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int z = z0 + lane + 32 * r;
+    if (z < Nz) {
+      float4* dst = reinterpret_cast<float4*>(sP + z * kTzfP);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) dst[q] = make_float4(ar[r][2 * q], ai[r][2 * q], ar[r][2 * q + 1], ai[r][2 * q + 1]);
+    }
+  }
+}
+
+template <bool V4>
+__global__ void __launch_bounds__(256, 3)
     k_fwd_tz_f32(const float* __restrict__ in, float2* __restrict__ out, long long ncol, int Nz,
-                 int Nt, int Jz, int Jt, const float2* __restrict__ ft,
-                 const float2* __restrict__ fz) {
+                 int Nt, int mz, int Jt, const float2* __restrict__ ft, const float2* __restrict__ fz) {
   extern __shared__ float4 smem4[];
-  float2* sFt = reinterpret_cast<float2*>(smem4);  // [Jt][Nt]
-  float2* sFz = sFt + Jt * Nt;                      // [Jz][Nz + 1]
-  float2* sP = sFz + Jz * (Nz + 1);                 // [Nz][Jt]
-  for (int e = threadIdx.x; e < Jt * Nt; e += blockDim.x) sFt[e] = ft[e];
-  for (int e = threadIdx.x; e < Jz * Nz; e += blockDim.x) {
-    int r = e / Nz, c = e - r * Nz;
-    sFz[r * (Nz + 1) + c] = fz[e];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const int J8 = (Jt + 7) / 8, TH = Nt / 2 + 1, ZH = Nz / 2 + 1, KP = mz + 1, Jz = 2 * mz;
+  const int CR = V4 ? 64 : tzf_rows_at_once(Nz, Nt);
+  const size_t colf = V4 ? 0 : (((size_t)min(Nz, CR) * Nt + 3) & ~(size_t)3);
+  float2* sF = reinterpret_cast<float2*>(smem4);  // [J8][TH][8] (cos, -sin) * scale
+  float2* sZ = sF + J8 * TH * 8;                  // [ZH][KP] (cos, sin) of k z
+  float2* sP = sZ + ((ZH * KP + 1) & ~1) + (size_t)warp * (kTzfP * Nz + colf / 2);  // [Nz][kTzfP]
+  float* sX = reinterpret_cast<float*>(sP + kTzfP * Nz);                            // [CR][Nt] (not V4)
+  for (int e = threadIdx.x; e < J8 * TH * 8; e += blockDim.x) {
+    const int q = e % 8, t = (e / 8) % TH, j = 8 * (e / (8 * TH)) + q;
+    sF[e] = j < Jt ? ft[(long long)j * Nt + t] : make_float2(0.f, 0.f);
+  }
+  for (int e = threadIdx.x; e < ZH * KP; e += blockDim.x) {
+    const int k = e % KP, z = e / KP;
+    const float2 f = fz[(long long)k * Nz + z];  // k < mz: exp(-i k z); k = mz: stored as -mz
+    sZ[e] = make_float2(f.x, k < mz ? -f.y : f.y);
   }
   __syncthreads();
-  const int JZT = Jz * Jt;
-  for (long long col = blockIdx.x; col < ncol; col += gridDim.x) {
+  const int jt = lane & 7, kg = lane >> 3;
+  for (long long col = (long long)blockIdx.x * W + warp; col < ncol; col += (long long)gridDim.x * W) {
     const float* src = in + col * (long long)Nz * Nt;
-    for (int z = threadIdx.x; z < Nz; z += blockDim.x) {
-      const float* row = src + (long long)z * Nt;
-      for (int j0 = 0; j0 < Jt; j0 += 8) {
-        float ar[8], ai[8];
+    for (int j8 = 0; j8 < J8; ++j8) {
+      const float2* F = sF + j8 * TH * 8;
+      for (int z0 = 0; z0 < Nz; z0 += CR) {
+        const float* rows = src;
+        if (!V4) {
+          const int n = min(CR, Nz - z0) * Nt;
+          const float* from = src + (long long)z0 * Nt;
+          __syncwarp();
+          for (int e0 = lane; e0 < n; e0 += 32 * 8) {
+            float v[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) { ar[q] = 0.f; ai[q] = 0.f; }
-        if (VEC4) {
-          for (int t = 0; t < Nt; t += 4) {
-            float4 v4 = __ldg(reinterpret_cast<const float4*>(row + t));
-            float vv[4] = {v4.x, v4.y, v4.z, v4.w};
+            for (int u = 0; u < 8; ++u) v[u] = e0 + 32 * u < n ? __ldg(from + e0 + 32 * u) : 0.f;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                if (j0 + q < Jt) {
-                  float2 f = sFt[(j0 + q) * Nt + t + u];
-                  ar[q] = fmaf(vv[u], f.x, ar[q]);
-                  ai[q] = fmaf(vv[u], f.y, ai[q]);
-                }
-              }
-            }
+            for (int u = 0; u < 8; ++u)
+              if (e0 + 32 * u < n) sX[e0 + 32 * u] = v[u];
           }
-        } else {
-          for (int t = 0; t < Nt; ++t) {
-            float v = __ldg(row + t);
+          __syncwarp();
+          rows = sX - (long long)z0 * Nt;
+        }
+        if (CR == 64 && Nz - z0 > 32)
+          tzf_rows<V4, 2>(rows, sP, F, z0, Nz, Nt, lane);
+        else
+          tzf_rows<V4, 1>(rows, sP, F, z0, Nz, Nt, lane);
+      }
+      __syncwarp();
+      const float2* P = sP + jt;
+      const int j = 8 * j8 + jt;
+      float2* dst = out + col * (long long)(Jz * Jt) + j;
+      for (int kc = 0; kc < KP; kc += 12) {
+        float2 A[3], Bs[3];  // sums over cosines and sines, (re, im)
+        const float2* f0[3];
+        const float2 p0 = P[0];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              if (j0 + q < Jt) {
-                float2 f = sFt[(j0 + q) * Nt + t];
-                ar[q] = fmaf(v, f.x, ar[q]);
-                ai[q] = fmaf(v, f.y, ai[q]);
-              }
-            }
+        for (int r = 0; r < 3; ++r) {
+          f0[r] = sZ + min(kc + kg + 4 * r, KP - 1);
+          A[r] = p0;
+          Bs[r] = make_float2(0.f, 0.f);
+        }
+#pragma unroll 4
+        for (int z = 1; 2 * z < Nz; ++z) {
+          const float2 a = P[z * kTzfP], b = P[(Nz - z) * kTzfP];
+          const float sr = a.x + b.x, si = a.y + b.y, dr = a.x - b.x, di = a.y - b.y;
+#pragma unroll
+          for (int r = 0; r < 3; ++r) {
+            const float2 f = f0[r][z * KP];
+            A[r].x = fmaf(f.x, sr, A[r].x);
+            A[r].y = fmaf(f.x, si, A[r].y);
+            Bs[r].x = fmaf(f.y, dr, Bs[r].x);
+            Bs[r].y = fmaf(f.y, di, Bs[r].y);
+          }
+        }
+        if (Nz % 2 == 0) {
+          const float2 a = P[(Nz / 2) * kTzfP];
+#pragma unroll
+          for (int r = 0; r < 3; ++r) {
+            const float c = f0[r][(Nz / 2) * KP].x;
+            A[r].x = fmaf(c, a.x, A[r].x);
+            A[r].y = fmaf(c, a.y, A[r].y);
           }
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (j0 + q < Jt) sP[z * Jt + j0 + q] = make_float2(ar[q], ai[q]);
+        for (int r = 0; r < 3; ++r) {
+          const int k = kc + kg + 4 * r;
+          if (j < Jt && k < KP) {
+            if (k < mz) dst[(long long)k * Jt] = make_float2(A[r].x + Bs[r].y, A[r].y - Bs[r].x);
+            if (k > 0) dst[(long long)(Jz - k) * Jt] = make_float2(A[r].x - Bs[r].y, A[r].y + Bs[r].x);
+          }
+        }
       }
+      __syncwarp();  // P (and the column) may be overwritten
     }
-    __syncthreads();
-    float2* dst = out + col * (long long)JZT;
-    for (int o = threadIdx.x; o < JZT; o += blockDim.x) {
-      int jz = o / Jt, jt = o - jz * Jt;
-      const float2* f = sFz + jz * (Nz + 1);
-      float re = 0.f, im = 0.f;
-      for (int z = 0; z < Nz; ++z) {
-        float2 a = f[z], b = sP[z * Jt + jt];
-        re = fmaf(a.x, b.x, re);
-        re = fmaf(-a.y, b.y, re);
-        im = fmaf(a.x, b.y, im);
-        im = fmaf(a.y, b.x, im);
-      }
-      dst[o] = make_float2(re, im);
-    }
-    __syncthreads();
   }
+}
+
+template <bool V4>
+static cudaError_t launch_tzf(const float* in, float2* out, int64_t ncol, const Dims& d, const float2* ft,
+                              const float2* fz, cudaStream_t s) {
+  int W = 8;  // fewer warps where their rows of P and columns do not fit two CTAs on an SM
+  while (W > 1 && tzf_smem(d, V4, W) > 110 * 1024) W /= 2;
+  const size_t smem = tzf_smem(d, V4, W);
+  const void* k = (const void*)k_fwd_tz_f32<V4>;
+  cudaError_t e = allow_smem(k, smem);
+  if (e != cudaSuccess) return e;
+  const int grid = persistent_grid(k, 32 * W, smem, (ncol + W - 1) / W);
+  FNO_LAUNCH("fno_fwd_tz_f32", k_fwd_tz_f32<V4>, grid, 32 * W, smem, s, in, out, (long long)ncol, (int)d.Nz,
+             (int)d.Nt, (int)d.mz, (int)d.Jt, ft, fz);
+  return cudaSuccess;
 }
 
 cudaError_t launch_fwd_tz_f32(const float* in, float2* out, int64_t ncol, const Dims& d,
                               const float2* ft, const float2* fz, cudaStream_t s) {
   if (ncol <= 0) return cudaSuccess;
-  size_t smem = fwd_tz_smem_bytes(d);
-  const int threads = 128;
-  if (d.Nt % 4 == 0) {
-    const void* k = (const void*)k_fwd_tz_f32<true>;
-    cudaError_t e = allow_smem(k, smem);
-    if (e != cudaSuccess) return e;
-    int grid = persistent_grid(k, threads, smem, ncol);
-    FNO_LAUNCH("fno_fwd_tz_f32", k_fwd_tz_f32<true>, grid, threads, smem, s, in, out,
-               (long long)ncol, (int)d.Nz, (int)d.Nt, (int)d.Jz, (int)d.Jt, ft, fz);
-  } else {
-    const void* k = (const void*)k_fwd_tz_f32<false>;
-    cudaError_t e = allow_smem(k, smem);
-    if (e != cudaSuccess) return e;
-    int grid = persistent_grid(k, threads, smem, ncol);
-    FNO_LAUNCH("fno_fwd_tz_f32", k_fwd_tz_f32<false>, grid, threads, smem, s, in, out,
-               (long long)ncol, (int)d.Nz, (int)d.Nt, (int)d.Jz, (int)d.Jt, ft, fz);
-  }
-  return cudaSuccess;
+  if (d.Nt % 4 == 0) return launch_tzf<true>(in, out, ncol, d, ft, fz, s);
+  return launch_tzf<false>(in, out, ncol, d, ft, fz, s);
 }
 
 // ---------------------------------------------------------------------------
