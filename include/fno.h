@@ -67,22 +67,24 @@ typedef struct fno_dims {
  *   FNO_BF16    BF16 tensor-core products (one product)
  *   FNO_BF16X3  split BF16 on the tensor cores: hi + lo with three products
  *               in the DFT stages, three-way splits with six products in the
- *               line stages and the mma.sync 1x1 stages; the 1x1 of the fused
- *               tcgen05 epilogue as 3xTF32 (big + small parts, three
- *               products), FP32-like
+ *               line stages; the 1x1 in FP32 (above 24 channels as 3xTF32 on
+ *               tcgen05: big + small parts, three products, FP32-like)
  * The tensor-core precisions need Nt even and at most 128, Nz * Nt a multiple
- * of 4, mt <= 8 and 2 mz <= 64 (FNO_ERR_UNSUPPORTED otherwise).  The fused
- * inverse z, t + epilogue stage runs, in FNO_BF16X3 and FNO_TF32, on tcgen05
- * (TMEM accumulators) for Nt = 16 or 32, Nz a multiple of 512 / Nt, 2 mz <= 24
- * and up to 32 channels; on warp-level mma.sync for FNO_BF16, the other shapes
- * its tiling takes and the dA pass of fno_block_bwd.  Other Nt (the paper's 84
- * and 86), with mt <= 8, up to 32 channels and the inverse z stage within the
- * tensor-core line tiling, take a synthesis path: the inverse z stage and the
- * inverse t stage to real points on mma.sync, the second written straight into
- * the output, then the 1x1, bias and GELU in FP32 in place (a workspace region
- * of B * max(C_in, C_out) * Nx * Ny * Nz * mt complex values holds the z stage;
- * the recomputing backward's dA pass stays on the FP32 kernel).  The FP32
- * kernels run the rest. */
+ * of 4, mt <= 8 and 2 mz <= 64 (FNO_ERR_UNSUPPORTED otherwise).  The inverse z, t +
+ * epilogue stage of FNO_BF16X3 is one kernel on warp-level mma.sync and packed
+ * FP32 (the column epilogue) with up to 32 channels, and on tcgen05 (TMEM
+ * accumulators) with more than 24 channels at Nt = 16 or 32, Nz a multiple of
+ * 512 / Nt, 2 mz <= 24.  FNO_TF32 runs on tcgen05 there with any channel count;
+ * FNO_BF16 on warp-level mma.sync (dX and the spectral form on the column
+ * epilogue); the dA pass of fno_block_bwd on mma.sync.  For other Nt (the paper's
+ * 84 and 86), with mt <= 8, up to 32 channels and the inverse z stage within the
+ * tensor-core line tiling, FNO_TF32 and FNO_BF16 (and grids of fewer than 32
+ * tiles of 16 planes) take a synthesis path: the inverse z stage and the inverse
+ * t stage to real points on mma.sync, the second written straight into the
+ * output, then the 1x1, bias and GELU in FP32 in place (a workspace region of B *
+ * max(C_in, C_out) * Nx * Ny * Nz * mt complex values holds the z stage and is
+ * part of the workspace at these Nt in every precision; the recomputing
+ * backward's dA pass stays on the FP32 kernel).  The FP32 kernels run the rest. */
 typedef enum fno_precision {
   FNO_FP32 = 0,
   FNO_TF32 = 1,
@@ -138,10 +140,10 @@ int fno_block_fwd(const fno_dims* dims, int precision, const float* x, const flo
  * floats), so that the fno_block_bwd_saved call after it forms dA = dz
  * GELU'(A) pointwise instead of evaluating the inverse transform and the 1x1
  * again (the derivative is the one of the erf form of GELU, Sec. IV-C's
- * block, taken at the forward's own A).  In the tensor-core precisions with
- * more than 31 input or 24 output channels (up to 32) re-evaluating A on the
- * tensor cores is the faster form: there the call skips the store and the
- * saved backward re-evaluates A, as after fno_block_fwd.  ws_bytes must cover
+ * block, taken at the forward's own A).  In FNO_BF16 and FNO_TF32 with more
+ * than 31 input or 24 output channels (up to 32) A is re-evaluated on the tensor
+ * cores instead: there the call skips the store and the saved backward
+ * re-evaluates A, as after fno_block_fwd. ws_bytes must cover
  * fno_workspace_bytes(dims, precision, FNO_OP_BLOCK_TRAIN) in every case; the
  * workspace is owned by the caller and must stay untouched until the
  * backward. */

@@ -421,11 +421,13 @@ static cudaError_t epilogue(const Dims& d, EpiArgs a, int precision, char* base,
 
 // Whether a training forward keeps GELU'(A) for the backward's dA pass.  The
 // pass wins wherever it contracts dW_lin on the tensor cores, and over the FP32
-// dA epilogue; with more channels than that in the tensor-core precisions, the
-// tensor-core dA epilogue (A re-evaluated from the kept spectra) is the faster
-// form, and the forward skips the store.
+// dA epilogue (32 channels, 2 x 64^3 x 32: 2284 us and 20 more in the forward,
+// against 4805 us for evaluating A again).  TF32 and plain BF16 beyond the two-CTA
+// form keep the evaluation: their gradients round dA, and an A that differs in its
+// last bit turns some of those roundings.
 static bool keep_gelu_grad(const Dims& d, int precision) {
   if (pointwise_da_mma_fits((int)d.Ci, (int)d.Co)) return true;
+  if (precision == FNO_BF16X3 && pointwise_da_mma_wide_fits((int)d.Ci, (int)d.Co)) return true;
   return !(is_tc(precision) &&
            epilogue_mma_supported(d, EPI_DA, (int)d.Co, (int)d.Ci, nullptr, 0));
 }

@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(kPwThreads, KB == 1 ? 4 : 1) k_pw_bwd(const Pw
 
 // ---------------------------------------------------------------------------
 // dA pass of a block backward after a training forward, with dW_lin and db on
-// the tensor cores, for C_in + 1 <= 32 rows and C_out <= 24
+// the tensor cores, for C_in + 1 <= 48 rows and C_out <= 32
 // ---------------------------------------------------------------------------
 // A tile is 256 points of one batch entry: rows of x, a row of ones, dz and
 // the saved GELU'(A), staged by cp.async.  Each thread forms dA = dz GELU'(A)
@@ -469,8 +469,15 @@ __global__ void __launch_bounds__(kPwThreads, KB == 1 ? 4 : 1) k_pw_bwd(const Pw
 // products start from zero (short accumulation chains) and are Kahan-folded
 // into per-thread sums; at the end the CTA adds its warps in a fixed order
 // into one row of partial sums.
-constexpr int kDaMT = 2;  // m-tiles of 16 over the C_in + 1 rows
-constexpr int kDaNT = 3;  // n-tiles of 8 over the C_out columns
+// TM m-tiles of 16 over the C_in + 1 rows, TN n-tiles of 8 over the C_out columns:
+// 2 x 3 with two CTAs on an SM, and 3 x 4 (up to 47 inputs and 32 outputs; one
+// CTA, whose sums take 144 registers) with two stages of up to 112 KB.  The wide
+// form takes 2284 us at 2 x 32 x 64^3 x 32 (8.6 GB: 0.55 of 6.8 TB/s); the FP32 pair
+// blocks took 6721, evaluating A again on the tensor cores 4805.  (A form without
+// staging, every warp loading its own 16 points of each channel, took 4014 there
+// and 2764 against 1537 us at 20 x 64^3 x 86: DRAM then serves 64-byte pieces of
+// sixty rows in turn.)
+constexpr int kDaMT = 2, kDaNT = 3, kDaMTWide = 3, kDaNTWide = 4;
 
 // a = big + small, both rounded to TF32 (nearest, ties away from zero; see
 // warp_mma.h)
@@ -487,8 +494,8 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-template <bool VEC>
-__global__ void __launch_bounds__(kPwThreads, 2) k_da_mma(const PwArgs k) {
+template <bool VEC, int TM, int TN>
+__global__ void __launch_bounds__(kPwThreads, TM * TN <= 6 ? 2 : 1) k_da_mma(const PwArgs k) {
   extern __shared__ __align__(16) float sm[];
   const int Ci = k.Ci, Co = k.Co;
   const int npair = Ci * Co + Co;
@@ -498,23 +505,23 @@ __global__ void __launch_bounds__(kPwThreads, 2) k_da_mma(const PwArgs k) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, c = lane & 3;
   const int MT = (Ci + 1 + 15) / 16, NT = (Co + 7) / 8;
-  float sum[kDaMT][kDaNT][4], cmp[kDaMT][kDaNT][4];
+  float sum[TM][TN][4], cmp[TM][TN][4];
 #pragma unroll
-  for (int m = 0; m < kDaMT; ++m)
+  for (int m = 0; m < TM; ++m)
 #pragma unroll
-    for (int n = 0; n < kDaNT; ++n)
+    for (int n = 0; n < TN; ++n)
 #pragma unroll
       for (int q = 0; q < 4; ++q) sum[m][n][q] = cmp[m][n][q] = 0.f;
   // fragment rows of x (clamped to the ones row; the extra rows are discarded)
   // and of dA (clamped to the last output; discarded likewise)
-  int xr[kDaMT][2], dr[kDaNT];
+  int xr[TM][2], dr[TN];
 #pragma unroll
-  for (int m = 0; m < kDaMT; ++m) {
+  for (int m = 0; m < TM; ++m) {
     xr[m][0] = min(16 * m + g, Ci) * kPwLd;
     xr[m][1] = min(16 * m + g + 8, Ci) * kPwLd;
   }
 #pragma unroll
-  for (int n = 0; n < kDaNT; ++n) dr[n] = min(8 * n + g, Co - 1) * kPwLd;
+  for (int n = 0; n < TN; ++n) dr[n] = min(8 * n + g, Co - 1) * kPwLd;
 
   const long long tpb = (k.P + kPwTile - 1) / kPwTile;
   const long long ntiles = k.B * tpb;
@@ -558,20 +565,20 @@ __global__ void __launch_bounds__(kPwThreads, 2) k_da_mma(const PwArgs k) {
       }
     }
     __syncthreads();  // the ones row and dA are in place
-    float acc[kDaMT][kDaNT][4];
+    float acc[TM][TN][4];
 #pragma unroll
-    for (int m = 0; m < kDaMT; ++m)
+    for (int m = 0; m < TM; ++m)
 #pragma unroll
-      for (int n = 0; n < kDaNT; ++n)
+      for (int n = 0; n < TN; ++n)
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
       const int k0 = 32 * warp + 8 * kk;
       if (k0 >= np) break;  // past the tile's end every operand is zero
-      uint32_t ab[kDaMT][4], as[kDaMT][4];
+      uint32_t ab[TM][4], as[TM][4];
 #pragma unroll
-      for (int m = 0; m < kDaMT; ++m) {
+      for (int m = 0; m < TM; ++m) {
         if (m < MT) {
           tf32_split(xs[xr[m][0] + k0 + c], ab[m][0], as[m][0]);
           tf32_split(xs[xr[m][1] + k0 + c], ab[m][1], as[m][1]);
@@ -580,13 +587,13 @@ __global__ void __launch_bounds__(kPwThreads, 2) k_da_mma(const PwArgs k) {
         }
       }
 #pragma unroll
-      for (int n = 0; n < kDaNT; ++n) {
+      for (int n = 0; n < TN; ++n) {
         if (n < NT) {
           uint32_t bb0, bs0, bb1, bs1;
           tf32_split(ds[dr[n] + k0 + c], bb0, bs0);
           tf32_split(ds[dr[n] + k0 + c + 4], bb1, bs1);
 #pragma unroll
-          for (int m = 0; m < kDaMT; ++m) {
+          for (int m = 0; m < TM; ++m) {
             if (m < MT) {
               mma_tf32(acc[m][n], as[m], bb0, bb1);
               mma_tf32(acc[m][n], ab[m], bs0, bs1);
@@ -597,9 +604,9 @@ __global__ void __launch_bounds__(kPwThreads, 2) k_da_mma(const PwArgs k) {
       }
     }
 #pragma unroll
-    for (int m = 0; m < kDaMT; ++m)
+    for (int m = 0; m < TM; ++m)
 #pragma unroll
-      for (int n = 0; n < kDaNT; ++n)
+      for (int n = 0; n < TN; ++n)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {  // Kahan: sum - cmp tracks the exact total
           const float yv = acc[m][n][e] - cmp[m][n][e];
@@ -614,9 +621,9 @@ __global__ void __launch_bounds__(kPwThreads, 2) k_da_mma(const PwArgs k) {
   cp_async_wait<0>();
   __syncthreads();
 #pragma unroll
-  for (int m = 0; m < kDaMT; ++m)
+  for (int m = 0; m < TM; ++m)
 #pragma unroll
-    for (int n = 0; n < kDaNT; ++n)
+    for (int n = 0; n < TN; ++n)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int i = 16 * m + g + 8 * (e >> 1), o = 8 * n + 2 * c + (e & 1);
@@ -978,12 +985,14 @@ cudaError_t launch_pointwise_bwd(const float* x, const float* w, const float* bi
 // tensor-core form of the pass (k_da_mma): staged rows, stages (two when two
 // CTAs per SM still fit), shared-memory bytes
 bool pointwise_da_mma_fits(int Ci, int Co) { return Ci + 1 <= 16 * kDaMT && Co <= 8 * kDaNT; }
+bool pointwise_da_mma_wide_fits(int Ci, int Co) { return Ci + 1 <= 16 * kDaMTWide && Co <= 8 * kDaNTWide; }
 static void da_mma_plan(int Ci, int Co, int& nstage, size_t& smem) {
   const size_t stage = sizeof(float) * (size_t)(Ci + 1 + 2 * Co) * kPwLd;
-  nstage = (2 * stage <= 110 * 1024) ? 2 : 1;
+  nstage = (2 * stage <= (size_t)(pointwise_da_mma_fits(Ci, Co) ? 110 : 226) * 1024) ? 2 : 1;
   smem = std::max(nstage * stage, sizeof(float) * (size_t)(kPwThreads / 32) * (Ci * Co + Co));
 }
 
+template <int TM, int TN>
 static cudaError_t launch_da_mma(const float* x, const float* g, const float* dz, float* da,
                                  float* part, int max_rows, int64_t B, int64_t P, int Ci, int Co,
                                  int* rows_out, cudaStream_t s) {
@@ -1002,8 +1011,8 @@ static cudaError_t launch_da_mma(const float* x, const float* g, const float* dz
   a.Co = Co;
   a.nstage = nstage;
   const long long ntiles = B * ((P + kPwTile - 1) / kPwTile);
-  const void* kv = reinterpret_cast<const void*>(k_da_mma<true>);
-  const void* ks = reinterpret_cast<const void*>(k_da_mma<false>);
+  const void* kv = reinterpret_cast<const void*>(k_da_mma<true, TM, TN>);
+  const void* ks = reinterpret_cast<const void*>(k_da_mma<false, TM, TN>);
   allow_smem(kv, smem);
   allow_smem(ks, smem);
   const int nb = std::min(pw_blocks_per_sm(kv, smem), pw_blocks_per_sm(ks, smem));
@@ -1012,9 +1021,9 @@ static cudaError_t launch_da_mma(const float* x, const float* g, const float* dz
   grid = std::min<long long>(grid, max_rows);
   if (grid < 1) grid = 1;
   if (rows_aligned(P, x, dz) && rows_aligned(P, g, nullptr))
-    FNO_LAUNCH("fno_da_saved", k_da_mma<true>, (int)grid, kPwThreads, smem, s, a);
+    FNO_LAUNCH("fno_da_saved", (k_da_mma<true, TM, TN>), (int)grid, kPwThreads, smem, s, a);
   else
-    FNO_LAUNCH("fno_da_saved", k_da_mma<false>, (int)grid, kPwThreads, smem, s, a);
+    FNO_LAUNCH("fno_da_saved", (k_da_mma<false, TM, TN>), (int)grid, kPwThreads, smem, s, a);
   *rows_out = (int)grid;
   return cudaSuccess;
 }
@@ -1023,7 +1032,9 @@ cudaError_t launch_pointwise_bwd_saved(const float* x, const float* g, const flo
                                        float* part, int max_rows, int64_t B, int64_t P, int Ci,
                                        int Co, int* rows_out, cudaStream_t s) {
   if (pointwise_da_mma_fits(Ci, Co))
-    return launch_da_mma(x, g, dz, da, part, max_rows, B, P, Ci, Co, rows_out, s);
+    return launch_da_mma<kDaMT, kDaNT>(x, g, dz, da, part, max_rows, B, P, Ci, Co, rows_out, s);
+  if (pointwise_da_mma_wide_fits(Ci, Co))
+    return launch_da_mma<kDaMTWide, kDaNTWide>(x, g, dz, da, part, max_rows, B, P, Ci, Co, rows_out, s);
   // wider layers: the FP32 pair-block contraction of k_pw_bwd
   const PwPlan pl = pw_plan(Ci, Co, true);
   PwArgs a{};
