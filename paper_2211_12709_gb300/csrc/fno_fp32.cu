@@ -802,6 +802,15 @@ cudaError_t launch_mix_adjoint_f32(const Dims& d, const float2* xh, const float2
 //       E_0 = U_0, E_k = U_k + U_-k, O_k = U_k - U_-k, E_mz = U_-mz, O_mz = -U_-mz
 //   per point and 4 outputs at a time (shared-memory vector broadcasts):
 //       A_o = bias_o + sum_jt (Qr[jt][o] c_jt(t) - Qi[jt][o] s_jt(t)) + sum_i W(i, o) L_i
+// Even Nt (EO, up to 8 kt and 32 inputs): with the even and the odd kt summed apart,
+// S(t) = E + O and S(t + Nt / 2) = E - O, so a thread owns the points t and t + Nt /
+// 2 of a plane: half of the inverse-t multiply-adds, and each weight and Q value
+// read once for two points (tiles are then 128 such pairs).  The dA mode keeps one
+// point per thread and forms the same two sums, so that it finds the forward's A
+// bit for bit.  Forward and dX at 2 x 20 x 64^3 x 16: 1252 and 994 us with one point
+// a thread (a shared-memory read per four multiply-adds), 1078 and 818 here; at 20
+// x 64^3 x 86 2874 and 2178, here 2265 and 1546.  Sizes whose pair tiles need more
+// than 56 KB of shared memory keep one point a thread.
 //   SPECTRAL: out = A (no bias, no linear term)   FWD: out = GELU(A)
 //   DA: out = dA = dz GELU'(A), and dW_lin / db partial sums   DX: out = A
 // ---------------------------------------------------------------------------
@@ -879,12 +888,14 @@ size_t epilogue_smem_bytes(const Dims& d, int mode, int Cs, int Cl) {
 
 int epilogue_max_grid() { return 1024; }
 
-template <int MODE, int CLM, int JTM>
+template <int MODE, int CLM, int JTM, bool EO>
 __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
   extern __shared__ float4 smem4[];
   const EpiArgs& a = k.a;
   const int Cs = a.Cs, Cl = (MODE == EPI_SPECTRAL) ? 0 : a.Cl;
-  const int Jz = k.Jz, Jt = k.Jt, Nz = k.Nz, Nt = k.Nt, mz = k.mz, P = k.P, CS4 = k.CS4;
+  constexpr bool TWO = EO && MODE != EPI_DA;  // two points (t, t + Nt / 2) per thread
+  const int Jz = k.Jz, Jt = k.Jt, Nz = k.Nz, mz = k.mz, P = k.P, CS4 = k.CS4;
+  const int Nt = TWO ? k.Nt / 2 : k.Nt;  // t positions of a tile's points
   const int PP = P + 1;
   unsigned char* base = reinterpret_cast<unsigned char*>(smem4);
   float4* eo = reinterpret_cast<float4*>(base + k.off[0]);
@@ -915,6 +926,7 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
   const int p = tid;
   int cur_t = -1;
   float itr[JTM], iti[JTM];
+  float osign = 1.f;  // EO, dA mode: the sign of the odd kt at this thread's t
 
   // EPI_DA: work items are (4x4 block of (i, o), point group) pairs, item
   // it = g * nblk + block.  KG point groups split the points when there are
@@ -935,7 +947,7 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
   }
 
   const long long plane = (long long)Nz * Nt;
-  const long long chan = k.NxNy * plane;
+  const long long chan = k.NxNy * (TWO ? 2 * plane : plane);
   const long long t_begin = k.ntiles * blockIdx.x / gridDim.x;
   const long long t_end = k.ntiles * (blockIdx.x + 1) / gridDim.x;
   long long cur_col = -1;
@@ -949,10 +961,12 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
     const long long b = col / k.NxNy, xy = col - b * k.NxNy;
     const int zz_p = (tf + p) / Nt, t = (tf + p) - zz_p * Nt;
     if (t != cur_t) {
+      const int tb = (EO && !TWO && t >= k.Nt / 2) ? t - k.Nt / 2 : t;
+      if (EO && !TWO) osign = tb == t ? 1.f : -1.f;
 #pragma unroll
       for (int jt = 0; jt < JTM; ++jt) {
         if (jt < Jt) {
-          const float2 f = __ldg(a.It + jt * Nt + t);
+          const float2 f = __ldg(a.It + jt * k.Nt + tb);
           itr[jt] = f.x;
           iti[jt] = -f.y;
         } else {
@@ -993,13 +1007,17 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
       __syncthreads();
     }
     // lin inputs of this point (issued early; consumed after Q is ready)
-    float x[CLM > 0 ? CLM : 1];
-    const long long pofs = xy * plane + s0 + p;
+    float x[CLM > 0 ? CLM : 1], x2[TWO && CLM > 0 ? CLM : 1];
+    const long long pofs =
+        TWO ? xy * 2 * plane + (long long)(z0 + zz_p) * k.Nt + t : xy * plane + s0 + p;
     const bool pv = p < valid;
     if (MODE != EPI_SPECTRAL) {
       const float* xp = a.lin_in + (b * Cl) * chan + pofs;
 #pragma unroll
-      for (int i = 0; i < CLM; ++i) x[i] = (i < Cl && pv) ? __ldg(xp + (long long)i * chan) : 0.f;
+      for (int i = 0; i < CLM; ++i) {
+        x[i] = (i < Cl && pv) ? __ldg(xp + (long long)i * chan) : 0.f;
+        if (TWO) x2[TWO ? i : 0] = (i < Cl && pv) ? __ldg(xp + (long long)i * chan + Nt) : 0.f;
+      }
     }
     // Q of this tile's planes: one (o, jt, zz) unit per step
     {
@@ -1054,16 +1072,25 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
           for (int q = 0; q < 4; ++q) dzq[q] = (c0 + q < Cs) ? __ldg(dzp + (long long)(c0 + q) * chan) : 0.f;
         }
         float4 acc = *reinterpret_cast<const float4*>(sbias + c0);
+        float4 odd = make_float4(0.f, 0.f, 0.f, 0.f);  // EO: the odd kt
 #pragma unroll
         for (int jt = 0; jt < JTM; ++jt) {
           if (jt < Jt) {
             const float4 qr = *reinterpret_cast<const float4*>(qp + (size_t)(jt * 2) * CS4 + c0);
             const float4 qi = *reinterpret_cast<const float4*>(qp + (size_t)(jt * 2 + 1) * CS4 + c0);
-            acc.x = fmaf(qr.x, itr[jt], fmaf(qi.x, iti[jt], acc.x));
-            acc.y = fmaf(qr.y, itr[jt], fmaf(qi.y, iti[jt], acc.y));
-            acc.z = fmaf(qr.z, itr[jt], fmaf(qi.z, iti[jt], acc.z));
-            acc.w = fmaf(qr.w, itr[jt], fmaf(qi.w, iti[jt], acc.w));
+            float4& s = (EO && (jt & 1)) ? odd : acc;
+            s.x = fmaf(qr.x, itr[jt], fmaf(qi.x, iti[jt], s.x));
+            s.y = fmaf(qr.y, itr[jt], fmaf(qi.y, iti[jt], s.y));
+            s.z = fmaf(qr.z, itr[jt], fmaf(qi.z, iti[jt], s.z));
+            s.w = fmaf(qr.w, itr[jt], fmaf(qi.w, iti[jt], s.w));
           }
+        }
+        float4 acc2 = acc;  // TWO: the point at t + Nt / 2
+        if (TWO) {
+          acc2 = make_float4(acc.x - odd.x, acc.y - odd.y, acc.z - odd.z, acc.w - odd.w);
+          acc = make_float4(acc.x + odd.x, acc.y + odd.y, acc.z + odd.z, acc.w + odd.w);
+        } else if (EO) {
+          acc = make_float4(acc.x + osign * odd.x, acc.y + osign * odd.y, acc.z + osign * odd.z, acc.w + osign * odd.w);
         }
         if (MODE != EPI_SPECTRAL) {
           const float* wp = sw + c0;
@@ -1074,9 +1101,17 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
             acc.y = fmaf(w4.y, x[i], acc.y);
             acc.z = fmaf(w4.z, x[i], acc.z);
             acc.w = fmaf(w4.w, x[i], acc.w);
+            if (TWO) {
+              const float v = x2[TWO ? i : 0];
+              acc2.x = fmaf(w4.x, v, acc2.x);
+              acc2.y = fmaf(w4.y, v, acc2.y);
+              acc2.z = fmaf(w4.z, v, acc2.z);
+              acc2.w = fmaf(w4.w, v, acc2.w);
+            }
           }
         }
         const float av[4] = {acc.x, acc.y, acc.z, acc.w};
+        const float av2[4] = {acc2.x, acc2.y, acc2.z, acc2.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int c = c0 + q;
@@ -1084,13 +1119,18 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
             float* o = optr + (long long)c * chan;
             if (MODE == EPI_FWD) {
               *o = gelu_f(av[q]);
-              if (a.gp) a.gp[o - a.out] = gelu_grad_f(av[q]);  // training forward
+              if (TWO) o[Nt] = gelu_f(av2[q]);
+              if (a.gp) {  // training forward
+                a.gp[o - a.out] = gelu_grad_f(av[q]);
+                if (TWO) a.gp[o - a.out + Nt] = gelu_grad_f(av2[q]);
+              }
             } else if (MODE == EPI_DA) {
               const float da = dzq[q] * gelu_grad_f(av[q]);
               *o = da;
               sda[c * PP + p] = da;
             } else {
               *o = av[q];
+              if (TWO) o[Nt] = av2[q];
             }
           } else if (MODE == EPI_DA && c < CS4) {
             sda[c * PP + p] = 0.f;
@@ -1180,13 +1220,24 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
   }
 }
 
-template <int MODE, int CLM, int JTM>
-static cudaError_t launch_epi_t(const Dims& d, const EpiArgs& a, int* grid_used, cudaStream_t s) {
+// Even Nt with two points per thread (see the top): by the sizes of the block
+// alone, so that the forward and the dA mode agree.
+static Dims half_t(Dims d) {
+  d.Nt /= 2;
+  return d;
+}
+static bool epi_even_odd(const Dims& d, int Cs, int Cl) {
+  return d.Nt % 2 == 0 && d.Jt <= 8 && Cl <= 32 && epilogue_smem_bytes(half_t(d), EPI_FWD, Cs, Cl) <= 56 * 1024;
+}
+
+template <int MODE, int CLM, int JTM, bool EO>
+static cudaError_t launch_epi_t(const Dims& d0, const EpiArgs& a, int* grid_used, cudaStream_t s) {
+  const Dims d = (EO && MODE != EPI_DA) ? half_t(d0) : d0;  // tiles of points or of pairs
   EpiK k{};
   k.a = a;
   k.NxNy = d.Nx * d.Ny;
   k.Nz = (int)d.Nz;
-  k.Nt = (int)d.Nt;
+  k.Nt = (int)d0.Nt;
   k.Jz = (int)d.Jz;
   k.Jt = (int)d.Jt;
   k.mz = (int)d.mz;
@@ -1206,7 +1257,7 @@ static cudaError_t launch_epi_t(const Dims& d, const EpiArgs& a, int* grid_used,
     for (int q = 0; q < 8; ++q) k.off[q] = (uint32_t)off[q];
   }
   const size_t smem = epilogue_smem_bytes(d, MODE, a.Cs, Cl);
-  const void* kern = (const void*)k_epi_f32<MODE, CLM, JTM>;
+  const void* kern = (const void*)k_epi_f32<MODE, CLM, JTM, EO>;
   cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int grid = persistent_grid(kern, 128, smem, k.ntiles);
@@ -1216,33 +1267,40 @@ static cudaError_t launch_epi_t(const Dims& d, const EpiArgs& a, int* grid_used,
                                  "fno_epi_dx_f32"};
   // the forward of a training step also stores GELU'(A)
   const char* name = (MODE == EPI_FWD && a.gp) ? "fno_epi_fwd_train_f32" : names[MODE];
-  FNO_LAUNCH(name, (k_epi_f32<MODE, CLM, JTM>), grid, 128, smem, s, k);
+  FNO_LAUNCH(name, (k_epi_f32<MODE, CLM, JTM, EO>), grid, 128, smem, s, k);
   return cudaSuccess;
 }
 
-template <int MODE, int JTM>
+template <int MODE, int JTM, bool EO>
 static cudaError_t launch_epi_j(const Dims& d, const EpiArgs& a, int* g, cudaStream_t s) {
   if constexpr (MODE == EPI_SPECTRAL) {
-    return launch_epi_t<MODE, 0, JTM>(d, a, g, s);
+    return launch_epi_t<MODE, 0, JTM, EO>(d, a, g, s);
   } else {
-  switch (epi_clm(a.Cl)) {
-    case 4: return launch_epi_t<MODE, 4, JTM>(d, a, g, s);
-    case 8: return launch_epi_t<MODE, 8, JTM>(d, a, g, s);
-    case 12: return launch_epi_t<MODE, 12, JTM>(d, a, g, s);
-    case 16: return launch_epi_t<MODE, 16, JTM>(d, a, g, s);
-    case 20: return launch_epi_t<MODE, 20, JTM>(d, a, g, s);
-    case 24: return launch_epi_t<MODE, 24, JTM>(d, a, g, s);
-    case 32: return launch_epi_t<MODE, 32, JTM>(d, a, g, s);
-    case 48: return launch_epi_t<MODE, 48, JTM>(d, a, g, s);
-    default: return launch_epi_t<MODE, 64, JTM>(d, a, g, s);
-  }
+    switch (epi_clm(a.Cl)) {
+      case 4: return launch_epi_t<MODE, 4, JTM, EO>(d, a, g, s);
+      case 8: return launch_epi_t<MODE, 8, JTM, EO>(d, a, g, s);
+      case 12: return launch_epi_t<MODE, 12, JTM, EO>(d, a, g, s);
+      case 16: return launch_epi_t<MODE, 16, JTM, EO>(d, a, g, s);
+      case 20: return launch_epi_t<MODE, 20, JTM, EO>(d, a, g, s);
+      case 24: return launch_epi_t<MODE, 24, JTM, EO>(d, a, g, s);
+      case 32: return launch_epi_t<MODE, 32, JTM, EO>(d, a, g, s);
+      default: break;
+    }
+    if constexpr (!EO) {
+      if (epi_clm(a.Cl) == 48) return launch_epi_t<MODE, 48, JTM, EO>(d, a, g, s);
+      return launch_epi_t<MODE, 64, JTM, EO>(d, a, g, s);
+    } else {
+      return cudaErrorInvalidValue;  // not reached: EO has at most 32 inputs
+    }
   }
 }
 
 template <int MODE>
 static cudaError_t launch_epi_m(const Dims& d, const EpiArgs& a, int* g, cudaStream_t s) {
-  if (d.Jt <= 8) return launch_epi_j<MODE, 8>(d, a, g, s);
-  return launch_epi_j<MODE, 16>(d, a, g, s);
+  const int Cl = MODE == EPI_SPECTRAL ? 0 : a.Cl;
+  if (epi_even_odd(d, a.Cs, Cl)) return launch_epi_j<MODE, 8, true>(d, a, g, s);
+  if (d.Jt <= 8) return launch_epi_j<MODE, 8, false>(d, a, g, s);
+  return launch_epi_j<MODE, 16, false>(d, a, g, s);
 }
 
 cudaError_t launch_epilogue_f32(const Dims& d, const EpiArgs& a, int* grid_used, cudaStream_t s) {
