@@ -557,9 +557,88 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// The same with two i a lane, 32 apart.  Shared-memory reads bound both forms (one
+// of the slab for each i and one of the table for each row, per 4 multiply-adds
+// and row), so a table value serves two i here.  Rows past nout repeat the last
+// one and are not stored.  Eight launches of a step: 20 x 64^3 x 32, modes
+// 12/12/8/8 455 us with one i, 354 with two; 2 x 20 x 64^3 x 16 422 and 404.
+static size_t line_pair_smem(int nin, int nout) {
+  return sizeof(float2) * (size_t)(nout * nin + nin * 64);
+}
+
+template <int QB>
+__global__ void __launch_bounds__(256)
+    k_line_pair_f32(const float2* __restrict__ in, float2* __restrict__ out, long long outer,
+                    int nin, int nout, long long inner, const float2* __restrict__ tab) {
+  extern __shared__ float4 smem4[];
+  float2* sTab = reinterpret_cast<float2*>(smem4);  // [nout][nin]
+  float2* sIn = sTab + nout * nin;                   // [nin][64]
+  const int lane = threadIdx.x, ty = threadIdx.y;
+  const int tid = ty * 32 + lane;
+  for (int e = tid; e < nout * nin; e += 256) sTab[e] = tab[e];
+  const long long ntile = (inner + 63) / 64;
+  const long long nwork = outer * ntile;
+  for (long long w = blockIdx.x; w < nwork; w += gridDim.x) {
+    const long long o = w / ntile;
+    const long long i = (w - o * ntile) * 64 + lane;
+    __syncthreads();
+    for (int n = ty; n < nin; n += 8)
+#pragma unroll
+      for (int v = 0; v < 2; ++v)
+        sIn[n * 64 + 32 * v + lane] =
+            i + 32 * v < inner ? in[(o * nin + n) * inner + i + 32 * v] : make_float2(0.f, 0.f);
+    __syncthreads();
+    for (int q0 = ty * QB; q0 < nout; q0 += 8 * QB) {
+      float2 acc[QB][2];
+      const float2* f[QB];
+#pragma unroll
+      for (int qq = 0; qq < QB; ++qq) {
+        f[qq] = sTab + min(q0 + qq, nout - 1) * nin;
+        acc[qq][0] = acc[qq][1] = make_float2(0.f, 0.f);
+      }
+#pragma unroll 4
+      for (int n = 0; n < nin; ++n) {
+        const float2 x[2] = {sIn[n * 64 + lane], sIn[n * 64 + 32 + lane]};
+#pragma unroll
+        for (int qq = 0; qq < QB; ++qq) {
+          const float2 t = f[qq][n];
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            acc[qq][v].x = fmaf(t.x, x[v].x, acc[qq][v].x);
+            acc[qq][v].x = fmaf(-t.y, x[v].y, acc[qq][v].x);
+            acc[qq][v].y = fmaf(t.x, x[v].y, acc[qq][v].y);
+            acc[qq][v].y = fmaf(t.y, x[v].x, acc[qq][v].y);
+          }
+        }
+      }
+#pragma unroll
+      for (int qq = 0; qq < QB; ++qq)
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+          if (q0 + qq < nout && i + 32 * v < inner)
+            out[(o * nout + q0 + qq) * inner + i + 32 * v] = acc[qq][v];
+    }
+  }
+}
+
 cudaError_t launch_line_f32(const float2* in, float2* out, int64_t outer, int nin, int nout,
                             int64_t inner, const float2* tab, cudaStream_t s) {
   if (outer <= 0 || inner <= 0) return cudaSuccess;
+  // Two i a lane where the tiles of 64 are hardly emptier than those of 32 (inner
+  // 96: a quarter of them idle), there are two for each SM, and four CTAs fit on
+  // one (64 -> 16 rows: 41 KB).  Axes that do not fit so keep one i a lane.
+  const int64_t t2 = (inner + 63) / 64, t1 = (inner + 31) / 32;
+  if (20 * t2 <= 11 * t1 && outer * t2 >= 2 * sm_count() &&
+      line_pair_smem(nin, nout) <= 56 * 1024) {
+    const size_t smem = line_pair_smem(nin, nout);
+    const void* k = (const void*)k_line_pair_f32<4>;
+    cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
+    const int grid = persistent_grid(k, 256, smem, outer * t2);
+    FNO_LAUNCH("fno_line_f32", k_line_pair_f32<4>, grid, dim3(32, 8), smem, s, in, out,
+               (long long)outer, nin, nout, (long long)inner, tab);
+    return cudaSuccess;
+  }
   size_t smem = line_smem_bytes(nin, nout);
   const void* k = (const void*)k_line_f32<4>;
   cudaError_t e = allow_smem(k, smem);
