@@ -185,16 +185,18 @@ def algorithmic(name, d):
 # which scales in proportion to the units processed.  An entry is removed when
 # its kernel changes.
 TRAFFIC_PER_UNIT = {
-    "fno_epi_fwd_train_f32": (0.804905e9 + 1.289400e9) / 167772160,
-    "fno_epi_da_f32": (1.476010e9 + 0.642174e9) / 167772160,
-    "fno_epi_dx_f32": (0.804837e9 + 0.609467e9) / 167772160,
+    "fno_fwd_tz_f32": (0.671154e9 + 0.114106e9) / 167772160,
+    "fno_epi_dx_cmma_bf16x3": (0.805722e9 + 0.611786e9) / 167772160,
+    "fno_epi_fwd_train_cmma_bf16x3": (0.805809e9 + 1.287845e9) / 167772160,
+    "fno_epi_fwd_train_f32": (0.804596e9 + 1.286313e9) / 167772160,
+    "fno_epi_dx_f32": (0.803867e9 + 0.609247e9) / 167772160,
     "fno_epi_da_mma_bf16x3": (1.471207e9 + 0.646687e9) / 167772160,
     "fno_epi_fwd_train_mma_bf16x3": (0.801008e9 + 1.291166e9) / 167772160,
     "fno_epi_dx_mma_bf16x3": (0.800973e9 + 0.613033e9) / 167772160,
-    "fno_fwd_tz_mma_bf16x3": (0.671138e9 + 0.108852e9) / 167772160,
+    "fno_fwd_tz_mma_bf16x3": (0.671133e9 + 0.112001e9) / 167772160,
     "fno_epi_fwd_train_tc_bf16x3": (0.798273e9 + 1.285392e9) / 167772160,
     "fno_epi_dx_tc_bf16x3": (0.798813e9 + 0.609447e9) / 167772160,
-    "fno_da_tz_bf16x3": (2.016318e9 + 0.765664e9) / 167772160,
+    "fno_da_tz_bf16x3": (2.015721e9 + 0.765448e9) / 167772160,
 }
 
 

@@ -32,15 +32,16 @@
 //   x staged by cp.async a unit ahead, 8 warps on an SM 9.62 ms
 //   three CTAs of 168 registers or four of 128          6.20 / 6.26 ms
 //   x loads before the z phase instead of after         6.08 ms
-//   every warp alone with the 1x1 on mma.sync (3xTF32)  9.27 ms
+//   every warp alone with the 1x1 on mma.sync (3xTF32)  9.25 ms
 // A packed FMA takes 2.3 cycles a scheduler, an mma.sync of this shape 8 (tf32
 // m16n8k8 as well, for half the products).  At Nt = 84 and 86 a unit has twelve
 // items, and what decides is L1: rows of 336 or 344 bytes share sectors and lines
 // between items.  Forward + dX at 262 x 118 x 64 x 86 and forward at 130^3 x 84:
 // two CTAs of six warps 18.4 and 12.4 ms, two of four 20.7 and 13.8, three of
 // four 22.1 and 17.8, one of eight 24.6 and 16.5 (synthesis path 34.0 and 20.7;
-// HBM asks for 10.4 and 6.6).  A third of the forward there goes into the partly
-// written sectors of the two stores.
+// HBM asks for 10.4 and 6.6).  A form that took 14 ms for the forward there took 9
+// with its two stores left out and no less without the loads of x: the partly
+// written sectors of 8-byte-aligned rows are the likely reason, not a measured one.
 //
 // Precision (accumulation FP32; the 1x1 is FP32, its operands rounded to BF16
 // before it where lin_round says so).  U, V and the bases enter as NP BF16
