@@ -5,7 +5,8 @@
 // Stage map (Alg. 2, Sec. IV-C of the paper; the forward truncated DFT runs
 // over the non-partitioned axes y, z, t first and over x last, the inverse is
 // the same chain in reverse order):
-//   k_fwd_tz_f32   pruned DFT over t then z of each (b, c, x, y) column
+//   k_fwd_tz_f32   pruned DFT over t then z of each (b, c, x, y) column, a warp each
+//   k_fwd_tz_cta_f32  the same with a CTA a column
 //   k_line_f32     one complex DFT axis (forward y, x; inverse x, y)
 //   k_mix_f32      per-mode complex channel mixing (the einsum of Alg. 2)
 //   k_mix_adj_f32  its adjoint: weight gradient and input-spectrum gradient
@@ -218,27 +219,34 @@ cudaError_t launch_tables(const Dims& d, const Tables& T, const EpiTables* et, i
 // Rows of a multiple of four floats are read straight from global memory, 16
 // bytes per lane; other rows are copied to shared memory as they lie, 32 or 64 at
 // a time (an odd row stride has no bank conflicts, Nt % 4 = 2 two-way ones; whole
-// columns of 22 KB left eight warps on an SM and took 4.27 ms at 20 x 64^3 x 86).
+// columns of 22 KB left eight warps on an SM and took 4.27 ms at 20 x 64^3 x 86), or
+// read 4 bytes at a time where the copies would leave few warps (tz_f32_form).
 // Issue bounds it.  One thread per row and per output with one basis read per two
 // multiply-adds took 641 us at 2 x 20 x 64^3 x 16 and 132 us at 2 x 12 x 45 x 37
 // x 27 x 21; this form 314 and 66 (three CTAs of 80 registers on an SM; two: 314
 // and 82).
 // ---------------------------------------------------------------------------
+// shared memory of the CTA form, which bounds the sizes that are accepted
 size_t fwd_tz_smem_bytes(const Dims& d) {
   return sizeof(float2) * (size_t)(d.Jt * d.Nt + d.Jz * (d.Nz + 1) + d.Nz * d.Jt);
 }
 
 constexpr int kTzfP = 10;  // float2 stride of a row of P (8 used): 16-byte stores without conflicts
 
-// rows copied at a time (not V4)
+// How a lane reads its rows: 16 bytes at a time (rows of a multiple of four
+// floats), from copied rows, or 4 bytes at a time where copies of 32 rows a warp
+// would leave few warps on an SM.
+enum TzfRows { TZF_VEC4, TZF_COPIED, TZF_DIRECT };
+
+// rows copied at a time (TZF_COPIED)
 __host__ __device__ inline int tzf_rows_at_once(int Nz, int Nt) { return Nz > 32 && Nt <= 32 ? 64 : 32; }
 
-// shared memory of W warps: tables, then per warp P and (not V4) the rows
-static size_t tzf_smem(const Dims& d, bool v4, int W) {
+// shared memory of W warps: tables, then per warp P and the copied rows
+static size_t tzf_smem(const Dims& d, TzfRows rows, int W) {
   const size_t tab = sizeof(float2) * ((size_t)((d.Jt + 7) / 8) * (d.Nt / 2 + 1) * 8 +
                                        (((size_t)(d.Nz / 2 + 1) * (d.mz + 1) + 1) & ~(size_t)1));
   const size_t col =
-      v4 ? 0 : sizeof(float) * (((size_t)std::min<int64_t>(d.Nz, tzf_rows_at_once((int)d.Nz, (int)d.Nt)) * d.Nt + 3) & ~(size_t)3);
+      rows != TZF_COPIED ? 0 : sizeof(float) * (((size_t)std::min<int64_t>(d.Nz, tzf_rows_at_once((int)d.Nz, (int)d.Nt)) * d.Nt + 3) & ~(size_t)3);
   return tab + (size_t)W * (sizeof(float2) * kTzfP * (size_t)d.Nz + col);
 }
 
@@ -380,19 +388,20 @@ __device__ __forceinline__ void tzf_rows(const float* __restrict__ src, float2* 
   }
 }
 
-template <bool V4>
+template <TzfRows ROWS>
 __global__ void __launch_bounds__(256, 3)
     k_fwd_tz_f32(const float* __restrict__ in, float2* __restrict__ out, long long ncol, int Nz,
                  int Nt, int mz, int Jt, const float2* __restrict__ ft, const float2* __restrict__ fz) {
   extern __shared__ float4 smem4[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
   const int J8 = (Jt + 7) / 8, TH = Nt / 2 + 1, ZH = Nz / 2 + 1, KP = mz + 1, Jz = 2 * mz;
-  const int CR = V4 ? 64 : tzf_rows_at_once(Nz, Nt);
-  const size_t colf = V4 ? 0 : (((size_t)min(Nz, CR) * Nt + 3) & ~(size_t)3);
+  constexpr bool V4 = ROWS == TZF_VEC4, COPY = ROWS == TZF_COPIED;
+  const int CR = COPY ? tzf_rows_at_once(Nz, Nt) : 64;
+  const size_t colf = !COPY ? 0 : (((size_t)min(Nz, CR) * Nt + 3) & ~(size_t)3);
   float2* sF = reinterpret_cast<float2*>(smem4);  // [J8][TH][8] (cos, -sin) * scale
   float2* sZ = sF + J8 * TH * 8;                  // [ZH][KP] (cos, sin) of k z
   float2* sP = sZ + ((ZH * KP + 1) & ~1) + (size_t)warp * (kTzfP * Nz + colf / 2);  // [Nz][kTzfP]
-  float* sX = reinterpret_cast<float*>(sP + kTzfP * Nz);                            // [CR][Nt] (not V4)
+  float* sX = reinterpret_cast<float*>(sP + kTzfP * Nz);                            // [CR][Nt] (COPY)
   for (int e = threadIdx.x; e < J8 * TH * 8; e += blockDim.x) {
     const int q = e % 8, t = (e / 8) % TH, j = 8 * (e / (8 * TH)) + q;
     sF[e] = j < Jt ? ft[(long long)j * Nt + t] : make_float2(0.f, 0.f);
@@ -410,7 +419,7 @@ __global__ void __launch_bounds__(256, 3)
       const float2* F = sF + j8 * TH * 8;
       for (int z0 = 0; z0 < Nz; z0 += CR) {
         const float* rows = src;
-        if (!V4) {
+        if (COPY) {
           const int n = min(CR, Nz - z0) * Nt;
           const float* from = src + (long long)z0 * Nt;
           __syncwarp();
@@ -480,26 +489,164 @@ __global__ void __launch_bounds__(256, 3)
   }
 }
 
-template <bool V4>
+// The same by a CTA of 128 threads per column, a thread per z row in the t stage and
+// per (jz, jt) output in the z stage, plain sums: a third of the shared memory on
+// long axes, and a column's rows in parallel.
+template <bool VEC4>
+__global__ void __launch_bounds__(128)
+    k_fwd_tz_cta_f32(const float* __restrict__ in, float2* __restrict__ out, long long ncol, int Nz,
+                     int Nt, int Jz, int Jt, const float2* __restrict__ ft,
+                     const float2* __restrict__ fz) {
+  extern __shared__ float4 smem4[];
+  float2* sFt = reinterpret_cast<float2*>(smem4);  // [Jt][Nt]
+  float2* sFz = sFt + Jt * Nt;                      // [Jz][Nz + 1]
+  float2* sP = sFz + Jz * (Nz + 1);                 // [Nz][Jt]
+  for (int e = threadIdx.x; e < Jt * Nt; e += blockDim.x) sFt[e] = ft[e];
+  for (int e = threadIdx.x; e < Jz * Nz; e += blockDim.x) {
+    int r = e / Nz, c = e - r * Nz;
+    sFz[r * (Nz + 1) + c] = fz[e];
+  }
+  __syncthreads();
+  const int JZT = Jz * Jt;
+  for (long long col = blockIdx.x; col < ncol; col += gridDim.x) {
+    const float* src = in + col * (long long)Nz * Nt;
+    for (int z = threadIdx.x; z < Nz; z += blockDim.x) {
+      const float* row = src + (long long)z * Nt;
+      for (int j0 = 0; j0 < Jt; j0 += 8) {
+        float ar[8], ai[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) { ar[q] = 0.f; ai[q] = 0.f; }
+        if (VEC4) {
+          for (int t = 0; t < Nt; t += 4) {
+            float4 v4 = __ldg(reinterpret_cast<const float4*>(row + t));
+            float vv[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                if (j0 + q < Jt) {
+                  float2 f = sFt[(j0 + q) * Nt + t + u];
+                  ar[q] = fmaf(vv[u], f.x, ar[q]);
+                  ai[q] = fmaf(vv[u], f.y, ai[q]);
+                }
+              }
+            }
+          }
+        } else {
+          for (int t = 0; t < Nt; ++t) {
+            float v = __ldg(row + t);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              if (j0 + q < Jt) {
+                float2 f = sFt[(j0 + q) * Nt + t];
+                ar[q] = fmaf(v, f.x, ar[q]);
+                ai[q] = fmaf(v, f.y, ai[q]);
+              }
+            }
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (j0 + q < Jt) sP[z * Jt + j0 + q] = make_float2(ar[q], ai[q]);
+      }
+    }
+    __syncthreads();
+    float2* dst = out + col * (long long)JZT;
+    for (int o = threadIdx.x; o < JZT; o += blockDim.x) {
+      int jz = o / Jt, jt = o - jz * Jt;
+      const float2* f = sFz + jz * (Nz + 1);
+      float re = 0.f, im = 0.f;
+      for (int z = 0; z < Nz; ++z) {
+        float2 a = f[z], b = sP[z * Jt + jt];
+        re = fmaf(a.x, b.x, re);
+        re = fmaf(-a.y, b.y, re);
+        im = fmaf(a.x, b.y, im);
+        im = fmaf(a.y, b.x, im);
+      }
+      dst[o] = make_float2(re, im);
+    }
+    __syncthreads();
+  }
+}
+
+// warps of a CTA of the warp-per-column form: fewer than eight where their rows of
+// P and their copied rows do not fit two CTAs on an SM
+static int tzf_warps(const Dims& d, TzfRows rows) {
+  int W = 8;
+  while (W > 1 && tzf_smem(d, rows, W) > 110 * 1024) W /= 2;
+  return W;
+}
+// warps of that form that an SM holds (0: not even one)
+static int tzf_warps_per_sm(const Dims& d, TzfRows rows) {
+  const int W = tzf_warps(d, rows);
+  const size_t smem = tzf_smem(d, rows, W);
+  if (smem > 227 * 1024) return 0;
+  return W * (int)std::min<size_t>(3, 228 * 1024 / (smem + 1024));
+}
+
+// Which form runs.  The plan of the warp-per-column form grows with Nz (80 bytes a
+// z row and warp) and, with copied rows, with Nt (32 rows a warp): the CTA form takes
+// every size whose warps do not fit, and what check_support admits is its plan.
+// Times in us at 1024 columns (256 where given), mt up to 8, warp / CTA form:
+//   16-byte rows: 1.1 to 2 times faster while an SM holds two warps (768 x 32: 172 /
+//     187; 512 x 1024, 256 columns: 543 / 704), slower with one (1024 x 16: 248 / 185;
+//     2500 x 8: 455 / 285).
+//   Copied rows: with 12 warps or more 10 / 12 (45 x 22) to 21 / 24 (64 x 86).  With
+//     fewer, short rows are faster read 4 bytes at a time, which keeps the copies out
+//     of shared memory (copied / direct / CTA: 262 x 22 43 / 23 / 49, 512 x 18 66 / 49 /
+//     86), unless one warp is left (1024 x 18 687 / 311 / 244).  Long rows thrash L1 that
+//     way (100 x 86: 31 / 58 / 56, 200 x 86: 168 / 217 / 144) and keep the copies down to
+//     six warps; with fewer, few planes leave L1 the room (32 x 510: 296 / 88 / 209), more
+//     do not (100 x 1022: 3032 / 1506 / 813).
+//   Long columns that are too few to give each scheduler a warp: 208 / 107 at 256
+//     columns of 64 x 1024, 227 / 103 at 130 x 512.
+enum TzForm { TZ_VEC4, TZ_COPIED, TZ_DIRECT, TZ_CTA };
+static TzForm tz_f32_form(const Dims& d, int64_t ncol) {
+  if (d.Nz > 48 && d.Nz * d.Nt >= 16384 && ncol < 4 * (int64_t)sm_count()) return TZ_CTA;
+  if (d.Nt % 4 == 0) return tzf_warps_per_sm(d, TZF_VEC4) >= 2 ? TZ_VEC4 : TZ_CTA;
+  if (tzf_warps_per_sm(d, TZF_COPIED) >= (d.Nt < 32 ? 12 : 6)) return TZ_COPIED;
+  if (d.Nt >= 32 && d.Nz > 48) return TZ_CTA;
+  return tzf_warps_per_sm(d, TZF_DIRECT) >= 2 ? TZ_DIRECT : TZ_CTA;
+}
+
+template <TzfRows ROWS>
 static cudaError_t launch_tzf(const float* in, float2* out, int64_t ncol, const Dims& d, const float2* ft,
                               const float2* fz, cudaStream_t s) {
-  int W = 8;  // fewer warps where their rows of P and columns do not fit two CTAs on an SM
-  while (W > 1 && tzf_smem(d, V4, W) > 110 * 1024) W /= 2;
-  const size_t smem = tzf_smem(d, V4, W);
-  const void* k = (const void*)k_fwd_tz_f32<V4>;
+  const int W = tzf_warps(d, ROWS);
+  const size_t smem = tzf_smem(d, ROWS, W);
+  const void* k = (const void*)k_fwd_tz_f32<ROWS>;
   cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) return e;
   const int grid = persistent_grid(k, 32 * W, smem, (ncol + W - 1) / W);
-  FNO_LAUNCH("fno_fwd_tz_f32", k_fwd_tz_f32<V4>, grid, 32 * W, smem, s, in, out, (long long)ncol, (int)d.Nz,
+  FNO_LAUNCH("fno_fwd_tz_f32", k_fwd_tz_f32<ROWS>, grid, 32 * W, smem, s, in, out, (long long)ncol, (int)d.Nz,
              (int)d.Nt, (int)d.mz, (int)d.Jt, ft, fz);
+  return cudaSuccess;
+}
+
+template <bool VEC4>
+static cudaError_t launch_tz_cta(const float* in, float2* out, int64_t ncol, const Dims& d, const float2* ft,
+                                 const float2* fz, cudaStream_t s) {
+  const size_t smem = fwd_tz_smem_bytes(d);
+  const void* k = (const void*)k_fwd_tz_cta_f32<VEC4>;
+  cudaError_t e = allow_smem(k, smem);
+  if (e != cudaSuccess) return e;
+  const int grid = persistent_grid(k, 128, smem, ncol);
+  FNO_LAUNCH("fno_fwd_tz_cta_f32", k_fwd_tz_cta_f32<VEC4>, grid, 128, smem, s, in, out, (long long)ncol, (int)d.Nz,
+             (int)d.Nt, (int)d.Jz, (int)d.Jt, ft, fz);
   return cudaSuccess;
 }
 
 cudaError_t launch_fwd_tz_f32(const float* in, float2* out, int64_t ncol, const Dims& d,
                               const float2* ft, const float2* fz, cudaStream_t s) {
   if (ncol <= 0) return cudaSuccess;
-  if (d.Nt % 4 == 0) return launch_tzf<true>(in, out, ncol, d, ft, fz, s);
-  return launch_tzf<false>(in, out, ncol, d, ft, fz, s);
+  switch (tz_f32_form(d, ncol)) {
+    case TZ_VEC4: return launch_tzf<TZF_VEC4>(in, out, ncol, d, ft, fz, s);
+    case TZ_COPIED: return launch_tzf<TZF_COPIED>(in, out, ncol, d, ft, fz, s);
+    case TZ_DIRECT: return launch_tzf<TZF_DIRECT>(in, out, ncol, d, ft, fz, s);
+    default: break;
+  }
+  if (d.Nt % 4 == 0) return launch_tz_cta<true>(in, out, ncol, d, ft, fz, s);
+  return launch_tz_cta<false>(in, out, ncol, d, ft, fz, s);
 }
 
 // ---------------------------------------------------------------------------
