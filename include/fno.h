@@ -277,13 +277,16 @@ int fno_adam_step(int64_t n, float* param, const float* grad, float* m, float* v
  *
  * fno_spectral_fwd_static computes exactly what fno_spectral_fwd computes, but
  * takes its scratch from a fixed array in the library's device memory
- * (FNO_STATIC_SCRATCH_BYTES = 16 MiB, held on every GPU that loads the library
- * until the process exits) instead of a caller workspace.  The caller still
+ * (FNO_STATIC_SCRATCH_BYTES = 16 MiB and 64 KiB more, held on every GPU that
+ * loads the library until the process exits) instead of a caller workspace.  The caller still
  * passes the input x, the weights w and the output y.  It calls no cudaMalloc,
  * cudaFree or other allocating routine.
  *   - Sizes whose fno_workspace_bytes(dims, precision, FNO_OP_SPECTRAL_FWD)
  *     exceeds FNO_STATIC_SCRATCH_BYTES are refused with FNO_ERR_UNSUPPORTED
- *     before anything is enqueued.
+ *     before anything is enqueued.  In FNO_BF16 and FNO_BF16X3 the basis
+ *     fragments of the column epilogue (at most 36 KiB of that size) are not
+ *     counted, so that sizes that much above are taken; the array's further 64
+ *     KiB hold them.
  *   - The first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress, with that device current); make that first call
  *     before capturing any stream.  The lookup also loads the library's device

@@ -198,7 +198,16 @@ static bool synth_region(const Dims& d) {
            epilogue_mma_supported(d, EPI_SPECTRAL, Ci, 0, nullptr, 0));
 }
 
-static Layout layout(const Dims& d, int op) {
+// whether a call of this precision may run the column epilogue, whose basis
+// fragments then have a place in the workspace (its modes take every channel count
+// that the spectral form takes, or fewer)
+static bool col_region(const Dims& d, int precision) {
+  return (precision == FNO_BF16X3 || precision == FNO_BF16) &&
+         (epilogue_col_supported(d, EPI_SPECTRAL, (int)d.Co, 0) ||
+          epilogue_col_supported(d, EPI_SPECTRAL, (int)d.Ci, 0));
+}
+
+static Layout layout(const Dims& d, int op, int precision) {
   Layout L{};
   size_t off = 0;
   L.err = off;
@@ -242,7 +251,8 @@ static Layout layout(const Dims& d, int op) {
   // a call runs one of the two
   L.tc_tab = off;
   L.epi_tab = off;
-  const size_t tcb = align256(epilogue_tc_table_bytes(d)), epb = align256(epi_tables_bytes(d));
+  const size_t tcb = align256(epilogue_tc_table_bytes(d));
+  const size_t epb = col_region(d, precision) ? align256(epi_tables_bytes(d)) : 0;
   L.extra = epb > tcb ? epb - tcb : 0;
   off += tcb + L.extra;
   if (op == FNO_OP_BLOCK_TRAIN) {
@@ -437,7 +447,7 @@ static int forward_common(const Dims& d, int precision, int op, const float* x, 
                           size_t ws_bytes, cudaStream_t s) {
   int rc = check_support(d, precision, op);
   if (rc) return rc;
-  const Layout L = layout(d, op);
+  const Layout L = layout(d, op, precision);
   if ((rc = check_ws(ws, ws_bytes, L))) return rc;
   REQ(w, 8);
   const bool block = (op == FNO_OP_BLOCK_FWD || op == FNO_OP_BLOCK_TRAIN);
@@ -559,7 +569,7 @@ size_t fno_workspace_bytes(const fno_dims* dims, int precision, int op) {
   Dims d;
   if (to_dims(dims, &d)) return 0;
   if (check_support(d, precision, op)) return 0;
-  return layout(d, op).total;
+  return layout(d, op, precision).total;
 }
 
 int fno_spectral_fwd(const fno_dims* dims, int precision, const float* x, const float* w,
@@ -607,7 +617,7 @@ int fno_spectral_bwd(const fno_dims* dims, int precision, const float* x, const 
   const int op = FNO_OP_SPECTRAL_BWD;
   saved_forget(ws);
   if ((rc = check_support(d, precision, op))) return rc;
-  const Layout L = layout(d, op);
+  const Layout L = layout(d, op, precision);
   if ((rc = check_ws(ws, ws_bytes, L))) return rc;
   if (!dx && !dw) return fail(FNO_ERR_INVALID_ARG, "dx and dw are both NULL");
   REQ(w, 8);
@@ -658,7 +668,7 @@ static int block_bwd_impl(const fno_dims* dims, int precision, const float* x, c
   if (rc) return rc;
   const int op = FNO_OP_BLOCK_BWD;
   if ((rc = check_support(d, precision, op))) return rc;
-  const Layout L = layout(d, op);
+  const Layout L = layout(d, op, precision);
   if ((rc = check_ws(ws, ws_bytes, L))) return rc;
   REQ(w, 8);
   REQ(w_lin, 4);
@@ -693,7 +703,7 @@ static int block_bwd_impl(const fno_dims* dims, int precision, const float* x, c
     return fail(FNO_ERR_INVALID_ARG,
                 "the workspace does not hold the state of an fno_block_fwd call with these "
                 "dims, precision, x and w");
-  const Layout LT = layout(d, FNO_OP_BLOCK_TRAIN);
+  const Layout LT = layout(d, FNO_OP_BLOCK_TRAIN, precision);
   if (train && (rc = check_ws(ws, ws_bytes, LT))) return rc;
   saved_forget(ws);  // the steps below overwrite the forward state
   CK(tables(d, base, L, T, EPI_DX, (int)d.Ci, (int)d.Co, precision, err, s));
@@ -958,8 +968,10 @@ int fno_profile_entry(int i, const char** name, int64_t* launches, double* total
 // file instead of a caller workspace (for callers that may not allocate device
 // memory; see include/fno.h).
 // ---------------------------------------------------------------------------
-// The limit of FNO_STATIC_SCRATCH_BYTES does not count Layout::extra (at most 24
-// KB of t fragments and 12 KB of z rows past Nz); the array has room for it.
+// The limit of FNO_STATIC_SCRATCH_BYTES does not count Layout::extra: in the
+// precisions and sizes of the column epilogue (even Nt <= 128, 2 mz <= 64) at most 24
+// KB of t fragments and 12 KB of z rows past Nz, else nothing.  The array has room
+// for it.
 static const size_t kStaticSlack = 64 * 1024;
 static __device__ __align__(256) unsigned char g_fno_static_scratch[FNO_STATIC_SCRATCH_BYTES + kStaticSlack];
 
@@ -1010,9 +1022,9 @@ extern "C" int fno_spectral_fwd_static(const fno_dims* dims, int precision, cons
   int rc = to_dims(dims, &d);
   if (rc) return rc;
   if ((rc = check_support(d, precision, FNO_OP_SPECTRAL_FWD))) return rc;
-  const Layout L = layout(d, FNO_OP_SPECTRAL_FWD);
+  const Layout L = layout(d, FNO_OP_SPECTRAL_FWD, precision);
   const size_t need = L.total - L.extra;
-  if (need > FNO_STATIC_SCRATCH_BYTES || L.extra > kStaticSlack)
+  if (need > FNO_STATIC_SCRATCH_BYTES)
     return fail(FNO_ERR_UNSUPPORTED,
                 "these sizes need %zu bytes of scratch; the static scratch holds %zu bytes "
                 "(use fno_spectral_fwd with a workspace)",
