@@ -429,15 +429,27 @@ static cudaError_t epilogue(const Dims& d, EpiArgs a, int precision, char* base,
   return launch_epilogue_f32(d, a, grid_used, s);
 }
 
+// Split BF16 beyond the two-CTA form of the dA pass (25..32 outputs or 32 inputs), on
+// the grids of k_epi_mma: the pass contracts dW_lin on the tensor cores in its wide
+// form, in place of the tensor-core dA epilogue, which evaluates A again (32
+// channels, 2 x 64^3 x 32: 2284 us and 20 more in the forward, against 4805).  Error of
+// dW_lin against 64 bits at 28 channels, 16 x 16 x 32 x 16: 3.3e-7 with that epilogue,
+// 2.8e-7 here.  In FP32, and on other grids, FP32 pair blocks form dW_lin: 2.3e-7
+// there (28 channels; this pass 2.6e-7), so they stay, though slower (64^3 x 16, 32
+// channels: 1692 us, against 579).
+static bool wide_da(const Dims& d, int precision) {
+  return precision == FNO_BF16X3 && !pointwise_da_mma_fits((int)d.Ci, (int)d.Co) &&
+         pointwise_da_mma_wide_fits((int)d.Ci, (int)d.Co) &&
+         epilogue_mma_supported(d, EPI_DA, (int)d.Co, (int)d.Ci, nullptr, 0);
+}
+
 // Whether a training forward keeps GELU'(A) for the backward's dA pass.  The
 // pass wins wherever it contracts dW_lin on the tensor cores, and over the FP32
-// dA epilogue (32 channels, 2 x 64^3 x 32: 2284 us and 20 more in the forward,
-// against 4805 us for evaluating A again).  TF32 and plain BF16 beyond the two-CTA
-// form keep the evaluation: their gradients round dA, and an A that differs in its
-// last bit turns some of those roundings.
+// dA epilogue.  TF32 and plain BF16 beyond the two-CTA form keep the evaluation:
+// their gradients round dA, and an A that differs in its last bit turns some of
+// those roundings.
 static bool keep_gelu_grad(const Dims& d, int precision) {
-  if (pointwise_da_mma_fits((int)d.Ci, (int)d.Co)) return true;
-  if (precision == FNO_BF16X3 && pointwise_da_mma_wide_fits((int)d.Ci, (int)d.Co)) return true;
+  if (pointwise_da_mma_fits((int)d.Ci, (int)d.Co) || wide_da(d, precision)) return true;
   return !(is_tc(precision) &&
            epilogue_mma_supported(d, EPI_DA, (int)d.Co, (int)d.Ci, nullptr, 0));
 }
@@ -727,7 +739,7 @@ static int block_bwd_impl(const fno_dims* dims, int precision, const float* x, c
       // dA = dz GELU'(A) from the training forward's GELU'(A): one pointwise
       // pass with the partial sums of dW_lin and db
       CK(launch_pointwise_bwd_saved(x, gp, dz, da, part, epilogue_max_grid(), d.B, d.Ng, (int)d.Ci, (int)d.Co,
-                                    &rows, s));
+                                    wide_da(d, precision), &rows, s));
     }
   } else {
   // dA = dz GELU'(A) with the partial sums of dW_lin and db

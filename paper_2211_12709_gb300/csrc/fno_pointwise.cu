@@ -37,9 +37,10 @@
 //
 // The block backward after a training forward uses the same staging for its
 // dA pass: dA = dz GELU'(A) from the forward's saved GELU'(A), written out,
-// with the (dW_lin, db) partial sums.  Up to 31 inputs and 24 outputs that
-// contraction runs on the tensor cores (k_da_mma, split TF32 products);
-// wider layers take the pair blocks of k_pw_bwd.
+// with the (dW_lin, db) partial sums.  Up to 31 inputs and 24 outputs, and up to 32
+// and 32 where its caller asks for it (split BF16), that contraction runs on the
+// tensor cores (k_da_mma, split TF32 products); wider layers take the FP32 pair
+// blocks of k_pw_bwd.
 #include <algorithm>
 
 #include "fno_internal.h"
@@ -453,7 +454,7 @@ __global__ void __launch_bounds__(kPwThreads, KB == 1 ? 4 : 1) k_pw_bwd(const Pw
 
 // ---------------------------------------------------------------------------
 // dA pass of a block backward after a training forward, with dW_lin and db on
-// the tensor cores, for C_in + 1 <= 48 rows and C_out <= 32
+// the tensor cores, for up to 32 inputs and 32 outputs
 // ---------------------------------------------------------------------------
 // A tile is 256 points of one batch entry: rows of x, a row of ones, dz and
 // the saved GELU'(A), staged by cp.async.  Each thread forms dA = dz GELU'(A)
@@ -470,10 +471,10 @@ __global__ void __launch_bounds__(kPwThreads, KB == 1 ? 4 : 1) k_pw_bwd(const Pw
 // into per-thread sums; at the end the CTA adds its warps in a fixed order
 // into one row of partial sums.
 // TM m-tiles of 16 over the C_in + 1 rows, TN n-tiles of 8 over the C_out columns:
-// 2 x 3 with two CTAs on an SM, and 3 x 4 (up to 47 inputs and 32 outputs; one
-// CTA, whose sums take 144 registers) with two stages of up to 112 KB.  The wide
-// form takes 2284 us at 2 x 32 x 64^3 x 32 (8.6 GB: 0.55 of 6.8 TB/s); the FP32 pair
-// blocks took 6721, evaluating A again on the tensor cores 4805.  (A form without
+// 2 x 3 with two CTAs on an SM (up to 31 inputs and 24 outputs), and 3 x 4 (up to 32
+// and 32; one CTA, whose sums take 144 registers) with two stages of up to 99 KB.  The
+// wide form takes 2284 us at 2 x 32 x 64^3 x 32 (8.6 GB: 0.55 of 6.8 TB/s); the FP32
+// pair blocks 6721, evaluating A again on the tensor cores 4805.  (A form without
 // staging, every warp loading its own 16 points of each channel, took 4014 there
 // and 2764 against 1537 us at 20 x 64^3 x 86: DRAM then serves 64-byte pieces of
 // sixty rows in turn.)
@@ -985,7 +986,7 @@ cudaError_t launch_pointwise_bwd(const float* x, const float* w, const float* bi
 // tensor-core form of the pass (k_da_mma): staged rows, stages (two when two
 // CTAs per SM still fit), shared-memory bytes
 bool pointwise_da_mma_fits(int Ci, int Co) { return Ci + 1 <= 16 * kDaMT && Co <= 8 * kDaNT; }
-bool pointwise_da_mma_wide_fits(int Ci, int Co) { return Ci + 1 <= 16 * kDaMTWide && Co <= 8 * kDaNTWide; }
+bool pointwise_da_mma_wide_fits(int Ci, int Co) { return Ci <= 32 && Co <= 8 * kDaNTWide; }
 static void da_mma_plan(int Ci, int Co, int& nstage, size_t& smem) {
   const size_t stage = sizeof(float) * (size_t)(Ci + 1 + 2 * Co) * kPwLd;
   nstage = (2 * stage <= (size_t)(pointwise_da_mma_fits(Ci, Co) ? 110 : 226) * 1024) ? 2 : 1;
@@ -1030,12 +1031,12 @@ static cudaError_t launch_da_mma(const float* x, const float* g, const float* dz
 
 cudaError_t launch_pointwise_bwd_saved(const float* x, const float* g, const float* dz, float* da,
                                        float* part, int max_rows, int64_t B, int64_t P, int Ci,
-                                       int Co, int* rows_out, cudaStream_t s) {
+                                       int Co, bool wide, int* rows_out, cudaStream_t s) {
   if (pointwise_da_mma_fits(Ci, Co))
     return launch_da_mma<kDaMT, kDaNT>(x, g, dz, da, part, max_rows, B, P, Ci, Co, rows_out, s);
-  if (pointwise_da_mma_wide_fits(Ci, Co))
+  if (wide && pointwise_da_mma_wide_fits(Ci, Co))
     return launch_da_mma<kDaMTWide, kDaNTWide>(x, g, dz, da, part, max_rows, B, P, Ci, Co, rows_out, s);
-  // wider layers: the FP32 pair-block contraction of k_pw_bwd
+  // the FP32 pair-block contraction of k_pw_bwd
   const PwPlan pl = pw_plan(Ci, Co, true);
   PwArgs a{};
   a.x = x;
