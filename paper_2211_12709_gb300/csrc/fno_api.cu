@@ -412,9 +412,11 @@ static cudaError_t epilogue(const Dims& d, EpiArgs a, int precision, char* base,
     case KIND_COL: {
       // on the grids that the fused forms tile, plain BF16 rounds the 1x1's
       // operands and split BF16 has three-product DFT stages; on the others the
-      // 1x1 is FP32 and split BF16 has six products
+      // 1x1 is FP32 and split BF16 has six products.  Where tcgen05 does not tile
+      // the grid, it stands in for the six-product 1x1 of k_epi_mma.
       const bool fused = epilogue_mma_supported(d, a.mode, a.Cs, a.Cl, nullptr, 0);
-      return launch_epilogue_col(d, a, split, !fused, fused && !split, epi_tables(d, base + L.epi_tab),
+      const bool fine = fused && !epilogue_tc_supported(d, a.mode, a.Cs, a.Cl, nullptr, 0);
+      return launch_epilogue_col(d, a, split, !fused, fused && !split, fine, epi_tables(d, base + L.epi_tab),
                                  a.It == tables_at(base, L).Its, s);
     }
     case KIND_TC:

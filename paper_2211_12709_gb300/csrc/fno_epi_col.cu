@@ -122,7 +122,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 
 // One t-phase item: the NPAIR channel pairs at this lane's points, H
 // sub-tiles of 8 points.
-template <int MODE, int CM, int NP, int H>
+template <int MODE, int CM, int NP, int H, int CH>
 __device__ __forceinline__ void col_item(const EpiCol& k, const uint4* sV, const uint4* sT, const ulonglong2* sW,
                                          const float2* sB, const u64 (&x)[CM > 0 ? CM : 1][H], char* out, char* gp,
                                          uint32_t pos, bool ok0, bool ok1) {
@@ -149,18 +149,20 @@ __device__ __forceinline__ void col_item(const EpiCol& k, const uint4* sV, const
         const uint4 f = A[P::a(q)], t = tb[P::b(q)];
         wm::mma16(s[h], f.x, f.y, f.z, f.w, h == 0 ? t.x : t.z, h == 0 ? t.y : t.w);
       }
-    // two chains of sums where the precision asks for it (NP = 3): one from the
-    // bias, one from S, half of the input channels each (z error at Nt = 84
-    // 1.29e-7 against 1.47e-7 in one chain, in the same time)
-    constexpr int IB = NP == 3 ? CM / 2 : CM;  // channels of the first chain
-    u64 a1[H], a2[H], b1[H], b2[H];
+    // the 1x1 in CH chains of FP32 sums, the first from the bias; S starts the second
+    // chain of several and is added to a single one
+    constexpr int K = CH > 2 ? CH : 2;
+    auto chain = [](int i) { return CH == 1 ? 0 : CH * i / CM; };
+    u64 a1[K][H], a2[K][H];
     const float2 bias = (MODE == EPI_FWD) ? sB[p] : make_float2(0.f, 0.f);
 #pragma unroll
     for (int h = 0; h < H; ++h) {
-      a1[h] = pack2(bias.x, bias.x);
-      a2[h] = pack2(bias.y, bias.y);
-      b1[h] = pack2(s[h][0], s[h][1]);
-      b2[h] = pack2(s[h][2], s[h][3]);
+      a1[0][h] = pack2(bias.x, bias.x);
+      a2[0][h] = pack2(bias.y, bias.y);
+      a1[1][h] = pack2(s[h][0], s[h][1]);
+      a2[1][h] = pack2(s[h][2], s[h][3]);
+#pragma unroll
+      for (int q = 2; q < K; ++q) a1[q][h] = a2[q][h] = 0;
     }
     if (MODE != EPI_SPECTRAL) {
       const ulonglong2* w = sW + p * CM;
@@ -169,22 +171,27 @@ __device__ __forceinline__ void col_item(const EpiCol& k, const uint4* sV, const
         const ulonglong2 wv = w[i];
 #pragma unroll
         for (int h = 0; h < H; ++h) {
-          fma2(i < IB ? a1[h] : b1[h], wv.x, x[i][h]);
-          fma2(i < IB ? a2[h] : b2[h], wv.y, x[i][h]);
+          fma2(a1[chain(i)][h], wv.x, x[i][h]);
+          fma2(a2[chain(i)][h], wv.y, x[i][h]);
         }
       }
     }
 #pragma unroll
     for (int h = 0; h < H; ++h) {
-      a1[h] = add2(a1[h], b1[h]);
-      a2[h] = add2(a2[h], b2[h]);
+#pragma unroll
+      for (int q = 2; q < K; ++q) {
+        a1[q - 2][h] = add2(a1[q - 2][h], a1[q][h]);
+        a2[q - 2][h] = add2(a2[q - 2][h], a2[q][h]);
+      }
+      a1[0][h] = add2(a1[0][h], a1[1][h]);
+      a2[0][h] = add2(a2[0][h], a2[1][h]);
     }
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       u64 z[H], d[H];
 #pragma unroll
       for (int h = 0; h < H; ++h) {
-        z[h] = c == 0 ? a1[h] : a2[h];
+        z[h] = c == 0 ? a1[0][h] : a2[0][h];
         if (MODE == EPI_FWD) gelu2(z[h], z[h], d[h]);
       }
       if (2 * p + c < Cs) {
@@ -211,8 +218,8 @@ __device__ __forceinline__ void col_item(const EpiCol& k, const uint4* sV, const
 }
 
 // CM: bound of the 1x1 input channels (register array), 0 for EPI_SPECTRAL.
-// H: sub-tiles of 8 t points of an item.
-template <int MODE, int CM, int NP, int H, int NW, int MINB>
+// H: sub-tiles of 8 t points of an item.  CH: chains of the 1x1's sums (1, 2, 4).
+template <int MODE, int CM, int NP, int H, int CH, int NW, int MINB>
 __global__ void __launch_bounds__(32 * NW, MINB) k_epi_col(const __grid_constant__ EpiCol k) {
   typedef Prods<NP> P;
   extern __shared__ __align__(16) unsigned char smem_col[];
@@ -395,7 +402,7 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_epi_col(const __grid_constant
             x[i][h] = pack2(lin_round(v.x, k.lin_round), lin_round(v.y, k.lin_round));
           }
       }
-      col_item<MODE, CM, NP, H>(k, sV + sub * NP * 32 + lane, sT + T * NP * 32 + lane, sW, sB, x, obase, gbase, pos,
+      col_item<MODE, CM, NP, H, CH>(k, sV + sub * NP * 32 + lane, sT + T * NP * 32 + lane, sW, sB, x, obase, gbase, pos,
                                 ok0, ok1);
       it += NW;
       if (it < nit) load_x(it);
@@ -413,52 +420,73 @@ bool epilogue_col_supported(const Dims& d, int mode, int Cs, int Cl) {
   return mode == EPI_SPECTRAL || (Cl >= 1 && Cl <= 32);
 }
 
-template <int MODE, int CM, int NP, int H, int NW, int MINB>
+template <int MODE, int CM, int NP, int H, int CH, int NW, int MINB>
 static cudaError_t launch_col_t(EpiCol k, const char* name, cudaStream_t s) {
   const int threads = 32 * NW;
   const size_t smem = sizeof(uint4) * (size_t)k.NPAIR * 2 * NP * 32 + sizeof(uint4) * (size_t)k.NTI * NP * 32 +
                       sizeof(ulonglong2) * (size_t)k.NPAIR * CM + sizeof(float2) * (size_t)((k.NPAIR + 1) & ~1) +
                       sizeof(float2) * (size_t)k.a.Cs * k.Jz * k.Jt;
-  const void* kern = (const void*)k_epi_col<MODE, CM, NP, H, NW, MINB>;
+  const void* kern = (const void*)k_epi_col<MODE, CM, NP, H, CH, NW, MINB>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
   const long long g = std::max<long long>(1, std::min<long long>((long long)per_sm * sm_count(), k.nunits));
-  FNO_LAUNCH(name, (k_epi_col<MODE, CM, NP, H, NW, MINB>), (int)g, threads, smem, s, k);
+  FNO_LAUNCH(name, (k_epi_col<MODE, CM, NP, H, CH, NW, MINB>), (int)g, threads, smem, s, k);
   return cudaSuccess;
 }
 
+// Chains of the 1x1's FP32 sums: one for plain BF16, two with three-part operands (z
+// error at Nt = 84 1.29e-7 against 1.47e-7 in one, in the same time).  With two parts
+// one chain of up to 24 channels is more exact than the tcgen05 form's 3xTF32 was
+// (z 1.6e-7 against 2.4e-7 at 20 channels); four chains are for what replaces the
+// six-product 1x1 of k_epi_mma (fine): z 1.61e-7 with one and 1.16e-7 with four
+// chains, 1.18e-7 in k_epi_mma, at 32 channels and Nt = 16, in the same time (32
+// channels: 488 us a dX either way at 64^3 x 16).  At 20 channels and Nt = 32 they
+// cost 4 to 7 %.
 template <int MODE, int NP>
-static cudaError_t launch_col_c(const EpiCol& k, bool narrow, const char* name, cudaStream_t s) {
-  if (MODE == EPI_SPECTRAL) {
-    if (narrow) return launch_col_t<EPI_SPECTRAL, 0, NP, 2, 4, 4>(k, name, s);
-    return launch_col_t<EPI_SPECTRAL, 0, NP, 1, 4, 4>(k, name, s);
+static cudaError_t launch_col_c(const EpiCol& k, bool narrow, bool fine, const char* name, cudaStream_t s) {
+  constexpr int C1 = NP == 3 ? 2 : 1, C4 = NP == 2 ? 4 : C1;
+  if constexpr (MODE == EPI_SPECTRAL) {
+    if (narrow) return launch_col_t<EPI_SPECTRAL, 0, NP, 2, 1, 4, 4>(k, name, s);
+    return launch_col_t<EPI_SPECTRAL, 0, NP, 1, 1, 4, 4>(k, name, s);
+  } else if (narrow) {
+    if (k.a.Cl <= 8) return launch_col_t<MODE, 8, NP, 2, C1, 4, 4>(k, name, s);
+    if (k.a.Cl <= 12) return launch_col_t<MODE, 12, NP, 2, C1, 4, 4>(k, name, s);
+    constexpr int NW = NP == 3 ? 6 : 4, MINB = NP == 3 ? 2 : 3;
+    if (k.a.Cl <= 20) {
+      if (fine) return launch_col_t<MODE, 20, NP, 2, C4, NW, MINB>(k, name, s);
+      return launch_col_t<MODE, 20, NP, 2, C1, NW, MINB>(k, name, s);
+    }
+    if (k.a.Cl <= 24) {
+      if (fine) return launch_col_t<MODE, 24, NP, 2, C4, NW, MINB>(k, name, s);
+      return launch_col_t<MODE, 24, NP, 2, C1, NW, MINB>(k, name, s);
+    }
+    return launch_col_t<MODE, 32, NP, 2, C4, 4, 2>(k, name, s);
+  } else {
+    if (k.a.Cl <= 8) return launch_col_t<MODE, 8, NP, 1, C1, 4, 5>(k, name, s);
+    if (k.a.Cl <= 20) {
+      if (fine) return launch_col_t<MODE, 20, NP, 1, C4, 4, 5>(k, name, s);
+      return launch_col_t<MODE, 20, NP, 1, C1, 4, 5>(k, name, s);
+    }
+    if (k.a.Cl <= 24) {
+      if (fine) return launch_col_t<MODE, 24, NP, 1, C4, 4, 4>(k, name, s);
+      return launch_col_t<MODE, 24, NP, 1, C1, 4, 4>(k, name, s);
+    }
+    return launch_col_t<MODE, 32, NP, 1, C4, 8, 2>(k, name, s);
   }
-  constexpr int M = MODE == EPI_SPECTRAL ? EPI_DX : MODE;
-  if (narrow) {
-    if (k.a.Cl <= 8) return launch_col_t<M, 8, NP, 2, 4, 4>(k, name, s);
-    if (k.a.Cl <= 12) return launch_col_t<M, 12, NP, 2, 4, 4>(k, name, s);
-    if (k.a.Cl <= 20) return launch_col_t<M, 20, NP, 2, NP == 3 ? 6 : 4, NP == 3 ? 2 : 3>(k, name, s);
-    if (k.a.Cl <= 24) return launch_col_t<M, 24, NP, 2, NP == 3 ? 6 : 4, NP == 3 ? 2 : 3>(k, name, s);
-    return launch_col_t<M, 32, NP, 2, 4, 2>(k, name, s);
-  }
-  if (k.a.Cl <= 8) return launch_col_t<M, 8, NP, 1, 4, 5>(k, name, s);
-  if (k.a.Cl <= 20) return launch_col_t<M, 20, NP, 1, 4, 5>(k, name, s);
-  if (k.a.Cl <= 24) return launch_col_t<M, 24, NP, 1, 4, 4>(k, name, s);
-  return launch_col_t<M, 32, NP, 1, 8, 2>(k, name, s);
 }
 
 template <int NP>
-static cudaError_t launch_col_m(const EpiCol& k, bool narrow, const char* name, cudaStream_t s) {
-  if (k.a.mode == EPI_SPECTRAL) return launch_col_c<EPI_SPECTRAL, NP>(k, narrow, name, s);
-  if (k.a.mode == EPI_DX) return launch_col_c<EPI_DX, NP>(k, narrow, name, s);
-  return launch_col_c<EPI_FWD, NP>(k, narrow, name, s);
+static cudaError_t launch_col_m(const EpiCol& k, bool narrow, bool fine, const char* name, cudaStream_t s) {
+  if (k.a.mode == EPI_SPECTRAL) return launch_col_c<EPI_SPECTRAL, NP>(k, narrow, fine, name, s);
+  if (k.a.mode == EPI_DX) return launch_col_c<EPI_DX, NP>(k, narrow, fine, name, s);
+  return launch_col_c<EPI_FWD, NP>(k, narrow, fine, name, s);
 }
 
 cudaError_t launch_epilogue_col(const Dims& d, const EpiArgs& a, bool split, bool exact, bool lin_round,
-                                const EpiTables& ct, bool scaled, cudaStream_t s) {
+                                bool fine, const EpiTables& ct, bool scaled, cudaStream_t s) {
   EpiCol k{};
   k.a = a;
   if (a.mode == EPI_SPECTRAL) k.a.Cl = 0;
@@ -484,9 +512,9 @@ cudaError_t launch_epilogue_col(const Dims& d, const EpiArgs& a, bool split, boo
                                           {"fno_epi_fwd_train_cmma_bf16", "fno_epi_fwd_train_cmma_bf16x3"}};
   const char* name = names[a.mode == EPI_SPECTRAL ? 0 : a.mode == EPI_DX ? 1 : a.gp ? 3 : 2][split ? 1 : 0];
   const bool narrow = ct.H == 2;
-  if (!split) return launch_col_m<1>(k, narrow, name, s);
-  if (exact) return launch_col_m<3>(k, narrow, name, s);
-  return launch_col_m<2>(k, narrow, name, s);
+  if (!split) return launch_col_m<1>(k, narrow, fine, name, s);
+  if (exact) return launch_col_m<3>(k, narrow, fine, name, s);
+  return launch_col_m<2>(k, narrow, fine, name, s);
 }
 
 }  // namespace fno

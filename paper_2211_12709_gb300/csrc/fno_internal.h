@@ -112,10 +112,11 @@ cudaError_t launch_epilogue_mma(const Dims& d, const EpiArgs& a, bool split, boo
 // (fno_epi_col.cu), modes EPI_FWD, EPI_DX and EPI_SPECTRAL, any even Nt <= 128;
 // same contract as launch_epilogue_f32 (no partial sums).  exact: split BF16 with
 // three parts and six products in the DFT stages (else two and three).
-// lin_round: the 1x1 operands rounded to BF16.  scaled: It is Its (else Itu).
+// lin_round: the 1x1 operands rounded to BF16.  fine: shorter chains of its sums
+// (not exact).  scaled: It is Its (else Itu).
 bool epilogue_col_supported(const Dims& d, int mode, int Cs, int Cl);
 cudaError_t launch_epilogue_col(const Dims& d, const EpiArgs& a, bool split, bool exact, bool lin_round,
-                                const EpiTables& ct, bool scaled, cudaStream_t s);
+                                bool fine, const EpiTables& ct, bool scaled, cudaStream_t s);
 
 // Inverse z, t + epilogue on the 5th-generation tensor cores (fno_tc.cu):
 // tcgen05.mma into TMEM accumulators, modes EPI_FWD, EPI_DX and EPI_SPECTRAL;
