@@ -804,7 +804,9 @@ cudaError_t launch_line_f32(const float2* in, float2* out, int64_t outer, int ni
 //            dw[i][o][j]  = sum_b conj(xh[b][i][j]) g[b][o][j]
 // A CTA owns a tile of kMixJ consecutive modes and has one group of kMixJ
 // threads per channel (output channels forward, input channels in the adjoint;
-// at most kMixG groups, which then take several in turn).  It stages the tile's
+// at most kMixG groups, which then take several in turn; kMixMin for fewer channels
+// with many rows to stage, the others helping there and, in the adjoint, sharing the
+// output channels of dW).  It stages the tile's
 // spectra for a chunk of BC batch entries in shared memory (rows of kMixJ
 // complex values: 128-byte coalesced loads), then each thread walks the summed
 // channel with kMixU weights in flight at a time, read straight from HBM in
@@ -816,10 +818,13 @@ cudaError_t launch_line_f32(const float2* in, float2* out, int64_t outer, int ni
 // forward and its adjoint took 59 and 57 us at 24576 modes, B = 2, width 20 (W 79
 // MB), here 27 and 42; 72 and 107, here 53 and 94 at 73728 modes, B = 1; 263 and
 // 361, here 207 and 354 at 110592 modes, B = 2, width 32.  20 weights in flight
-// measured slower (registers), 5 about as fast.
+// measured slower (registers), 5 about as fast.  One group and no more for a single
+// channel (20 -> 1 forward, 1 -> 20 adjoint, 24576 modes, B = 16) took 304 and 360 us,
+// 66 and 68 in 16 fixed groups, 60 and 75 here (mix_widen).
 // ---------------------------------------------------------------------------
 constexpr int kMixJ = 16;  // modes per tile
-constexpr int kMixG = 32;  // most channel groups of a CTA
+constexpr int kMixG = 32;    // most channel groups of a CTA
+constexpr int kMixMin = 16;  // groups where many rows are staged for few channels
 constexpr int kMixU = 10;  // weights in flight per thread
 
 __device__ __forceinline__ void cmac(float2& acc, const float2 a, const float2 b) {
@@ -867,7 +872,7 @@ __global__ void __launch_bounds__(kMixJ * kMixG, 2)
   for (int b0 = 0; b0 < B; b0 += BC) {
     const int nb = min(BC, B - b0);
     float2 wv[kMixU];
-    mix_load(wv, w + (long long)grp * Mk + j, step, 0, Ci, inj);
+    mix_load(wv, w + (long long)grp * Mk + j, step, 0, Ci, inj && grp < Co);
     __syncthreads();
     mix_stage(xs, xh, b0, nb, BC, Ci, Mk, j0);
     __syncthreads();
@@ -894,34 +899,38 @@ __global__ void __launch_bounds__(kMixJ * kMixG, 2)
   }
 }
 
-template <int BC>
+// SPLIT: several groups of threads per input channel, which share dW's outputs
+template <int BC, bool SPLIT>
 __global__ void __launch_bounds__(kMixJ * kMixG, 2)
     k_mix_adj_f32(const float2* __restrict__ xh, const float2* __restrict__ w,
                   const float2* __restrict__ g, float2* __restrict__ dw, float2* __restrict__ gxh,
-                  int B, int Ci, int Co, long long Mk) {
+                  int B, int Ci, int Co, long long Mk, int GI) {
   extern __shared__ float2 mix_sm[];
   float2* xs = mix_sm;                   // [BC][Ci][kMixJ]
   float2* gs = mix_sm + BC * Ci * kMixJ; // [BC][Co][kMixJ]
-  const int jl = threadIdx.x % kMixJ, grp = threadIdx.x / kMixJ, ngrp = blockDim.x / kMixJ;
+  // group (gi, go): input channels gi, gi + GI, ..; dW's outputs go, go + GO, ..
+  const int jl = threadIdx.x % kMixJ, grp = threadIdx.x / kMixJ;
+  const int GO = SPLIT ? blockDim.x / (kMixJ * GI) : 1;
+  const int gi = SPLIT ? grp % GI : grp, go = SPLIT ? grp / GI : 0;
   const long long j0 = (long long)blockIdx.x * kMixJ, j = j0 + jl;
   const bool inj = j < Mk;
   for (int b0 = 0; b0 < B; b0 += BC) {
     const int nb = min(BC, B - b0);
     float2 wv[kMixU];
-    mix_load(wv, w + (long long)grp * Co * Mk + j, Mk, 0, Co, inj && gxh);
+    mix_load(wv, w + (long long)gi * Co * Mk + j, Mk, 0, Co, inj && gxh && go == 0);
     __syncthreads();
     if (dw) mix_stage(xs, xh, b0, nb, BC, Ci, Mk, j0);
     mix_stage(gs, g, b0, nb, BC, Co, Mk, j0);
     __syncthreads();
     if (!inj) continue;
-    if (gxh) {
-      for (int i = grp; i < Ci; i += ngrp) {
+    if (gxh && go == 0) {
+      for (int i = gi; i < Ci; i += GI) {
         float2 ga[BC];
 #pragma unroll
         for (int q = 0; q < BC; ++q) ga[q] = make_float2(0.f, 0.f);
         const float2* wp = w + (long long)i * Co * Mk + j;
         for (int o0 = 0; o0 < Co; o0 += kMixU) {
-          if (o0 > 0 || i != grp) mix_load(wv, wp, Mk, o0, Co, true);
+          if (o0 > 0 || i != gi) mix_load(wv, wp, Mk, o0, Co, true);
 #pragma unroll
           for (int u = 0; u < kMixU; ++u) {
             if (o0 + u < Co) {
@@ -937,13 +946,13 @@ __global__ void __launch_bounds__(kMixJ * kMixG, 2)
     }
     // dW after it: reads of W and writes of dW in one loop measured slower
     if (dw) {
-      for (int i = grp; i < Ci; i += ngrp) {
+      for (int i = gi; i < Ci; i += GI) {
         float2 xv[BC];
 #pragma unroll
         for (int q = 0; q < BC; ++q) xv[q] = xs[(q * Ci + i) * kMixJ + jl];
-        float2* dp = dw + (long long)i * Co * Mk + j;
+        float2* dp = dw + ((long long)i * Co + go) * Mk + j;
 #pragma unroll 4
-        for (int o = 0; o < Co; ++o, dp += Mk) {
+        for (int o = go; o < Co; o += GO, dp += GO * Mk) {
           float2 da = make_float2(0.f, 0.f);
 #pragma unroll
           for (int q = 0; q < BC; ++q) cmac_conj(da, xv[q], gs[(q * Co + o) * kMixJ + jl]);
@@ -959,10 +968,32 @@ __global__ void __launch_bounds__(kMixJ * kMixG, 2)
   }
 }
 
-// Input-channel groups of the adjoint: one each up to 24 channels, else two in
-// turn (32 channels, B = 2: 330 us in 16 groups, 371 in 32; 20 channels: 46 in 16,
-// 38 in 20).
-static int mix_adj_groups(int64_t Ci) { return (int)(Ci <= 24 ? Ci : (Ci + 1) / 2); }
+// Channel groups of a CTA: one per channel up to 24 and, in the forward, 32; otherwise
+// two channels in turn.  21 to 24 groups put two CTAs of 64-register threads on an SM where
+// half as many put five: taken where the tiles fill the chip (24 channels, 73728
+// modes, B = 2: forward 104 us in 24 groups, 90 in 12; adjoint 177 and 154), not on
+// few tiles (2048 modes: 8.1 and 10.4, 10.9 and 14.3) and not in the adjoint with
+// eight batch entries at a time (B = 16: 810 and 893).  Other widths, adjoint: 32 at B
+// = 2 330 us in 16 groups, 371 in 32; 20 46 in 16, 38 in 20.
+static bool mix_halve(int64_t C, unsigned tiles) { return C >= 21 && C <= 24 && tiles >= 4u * (unsigned)sm_count(); }
+static int mix_groups(int64_t Co, unsigned tiles) {
+  return mix_halve(Co, tiles) ? (int)(Co + 1) / 2 : (int)std::min<int64_t>(kMixG, Co);
+}
+static int mix_adj_groups(int64_t Ci, int BC, unsigned tiles) {
+  if (Ci > 32 || (BC <= 4 && mix_halve(Ci, tiles))) return (int)(Ci + 1) / 2;
+  return Ci <= 24 ? (int)Ci : 16;
+}
+
+// Whether a CTA of `groups` groups takes kMixMin of them instead: so many rows to
+// stage that its few threads would take longer over them than over the sums.  Many
+// tiles hide the staging of one CTA behind others, so the line lies higher there
+// (rows a group, us without and with: 20, 128 tiles 12.3 / 6.7; 40, 1536 tiles 22.7 / 14.6,
+// 4608 tiles 30.4 / 33.3; 80, 4608 tiles 137 / 69).
+static bool mix_widen(int64_t rows, int groups, unsigned tiles) {
+  if (groups >= kMixMin) return false;
+  const unsigned sms = (unsigned)sm_count();
+  return rows > groups * (int64_t)(tiles < 4 * sms ? 8 : tiles < 16 * sms ? 32 : 44);
+}
 
 static int mix_bc(int64_t B) { return B <= 1 ? 1 : B <= 2 ? 2 : B <= 4 ? 4 : 8; }
 
@@ -975,8 +1006,10 @@ static cudaError_t launch_mix_bc(const Dims& d, const float2* xh, const float2* 
     if (e != cudaSuccess) return e;
   }
   const unsigned grid = (unsigned)((d.Mk + kMixJ - 1) / kMixJ);
-  FNO_LAUNCH("fno_mix_f32", k_mix_f32<BC>, grid, kMixJ * (int)std::min<int64_t>(kMixG, d.Co), smem, s, xh, w, yh, (int)d.B,
-             (int)d.Ci, (int)d.Co, (long long)d.Mk);
+  int groups = mix_groups(d.Co, grid);
+  if (mix_widen(BC * d.Ci, groups, grid)) groups = kMixMin;
+  FNO_LAUNCH("fno_mix_f32", k_mix_f32<BC>, grid, kMixJ * groups, smem, s, xh, w, yh, (int)d.B, (int)d.Ci,
+             (int)d.Co, (long long)d.Mk);
   return cudaSuccess;
 }
 
@@ -984,13 +1017,19 @@ template <int BC>
 static cudaError_t launch_mix_adj_bc(const Dims& d, const float2* xh, const float2* w,
                                      const float2* g, float2* dw, float2* gxh, cudaStream_t s) {
   const size_t smem = sizeof(float2) * (size_t)BC * (size_t)(d.Ci + d.Co) * kMixJ;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_mix_adj_f32<BC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
   const unsigned grid = (unsigned)((d.Mk + kMixJ - 1) / kMixJ);
-  FNO_LAUNCH("fno_mix_adjoint_f32", k_mix_adj_f32<BC>, grid, kMixJ * mix_adj_groups(d.Ci), smem, s, xh, w, g, dw,
-             gxh, (int)d.B, (int)d.Ci, (int)d.Co, (long long)d.Mk);
+  const int GI = mix_adj_groups(d.Ci, BC, grid);
+  const bool split = mix_widen(BC * (d.Co + (dw ? d.Ci : 0)), GI, grid);
+  const int threads = kMixJ * GI * (split ? kMixMin / GI : 1);
+  const void* k = split ? (const void*)k_mix_adj_f32<BC, true> : (const void*)k_mix_adj_f32<BC, false>;
+  cudaError_t e = allow_smem(k, smem);
+  if (e != cudaSuccess) return e;
+  if (split)
+    FNO_LAUNCH("fno_mix_adjoint_f32", (k_mix_adj_f32<BC, true>), grid, threads, smem, s, xh, w, g, dw, gxh, (int)d.B,
+               (int)d.Ci, (int)d.Co, (long long)d.Mk, GI);
+  else
+    FNO_LAUNCH("fno_mix_adjoint_f32", (k_mix_adj_f32<BC, false>), grid, threads, smem, s, xh, w, g, dw, gxh, (int)d.B,
+               (int)d.Ci, (int)d.Co, (long long)d.Mk, GI);
   return cudaSuccess;
 }
 
