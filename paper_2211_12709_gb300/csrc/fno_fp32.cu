@@ -1486,13 +1486,22 @@ __global__ void __launch_bounds__(128, 4) k_epi_f32(const EpiK k) {
 }
 
 // Even Nt with two points per thread (see the top): by the sizes of the block
-// alone, so that the forward and the dA mode agree.
+// alone, so that the forward and the dA mode agree.  Not where a column is one tile
+// either way, whose threads then are half idle (forward at 20 channels, 64 x 64 x 8 x
+// 4: 53 us with one point, 70 with two), and not where rows of an odd, small number of
+// pairs, which tiles cut, meet tiles that are not half as many and more than 12
+// channels (20 channels, 32 x 32 x 64 x 14: 176 and 195, spectral form 129 and 157; 24
+// at 64 x 32 x 64 x 10: 304 and 342; 4 at 64 x 64 x 64 x 10: 123 and 109).
 static Dims half_t(Dims d) {
   d.Nt /= 2;
   return d;
 }
 static bool epi_even_odd(const Dims& d, int Cs, int Cl) {
-  return d.Nt % 2 == 0 && d.Jt <= 8 && Cl <= 32 && epilogue_smem_bytes(half_t(d), EPI_FWD, Cs, Cl) <= 56 * 1024;
+  if (d.Nt % 2 != 0 || d.Jt > 8 || Cl > 32) return false;
+  const int64_t points = (d.Nz * d.Nt + kEpiP - 1) / kEpiP, pairs = (d.Nz * d.Nt / 2 + kEpiP - 1) / kEpiP;
+  if (pairs == points) return false;
+  if (2 * pairs > points && d.Nt < 16 && d.Nt % 4 != 0 && std::max(Cs, Cl) > 12) return false;
+  return epilogue_smem_bytes(half_t(d), EPI_FWD, Cs, Cl) <= 56 * 1024;
 }
 
 template <int MODE, int CLM, int JTM, bool EO>
