@@ -362,12 +362,16 @@ static cudaError_t synth_epilogue(const Dims& d, const EpiArgs& a, int precision
 
 // Which kernel runs the inverse z, t + epilogue stage of a call in the
 // tensor-core precisions (not the dA mode).  Times are forward + dX (us) of a
-// training step at 64^3 x Nt.
+// training step at 64^3 x Nt unless a grid is given.
 //   column epilogue (k_epi_col): split BF16, and dX and the spectral form in plain
 //     BF16 on the grids of k_epi_mma (the sums that it rounds run in the same
 //     order).  Against the tcgen05 kernel, Nt = 32: 294 : 931 at 8 channels, 688 :
 //     1005 at 16, 1280 : 1437 at 24; against the synthesis path, Nt = 86: 1047 :
 //     1860 at 8 channels, 502 : 1370 at 4, 5531 : 7881 at 32.
+//     Not where many of the planes of its tiles of 16 do not exist (col_thin), nor
+//     plain BF16 dX above 24 channels, where k_epi_mma is as fast or faster (dX alone,
+//     column form against it: 64^3 x 32 channels 246 : 220 at Nt = 16, 24 channels 73 : 70
+//     at 32 x 32 x 64 x 16; 64 x 64 x 8 x 16 at 28 channels 99 : 72).
 //   tcgen05 (k_epi_tc): beyond 24 channels, where its 32-wide products are full
 //     and the FP32 1x1 of the column form no longer is cheaper (Nt = 32, 32
 //     channels: 1502 : 1774; 24 channels: 1437 : 1280, at Nt = 16 807 : 721); and
@@ -376,9 +380,23 @@ static cudaError_t synth_epilogue(const Dims& d, const EpiArgs& a, int precision
 //     otherwise.  They keep their order of sums: dA and the spectra are
 //     rounded to 11 or 8 bits later, and a sum that differs in its last bit
 //     turns some of those roundings (rel 5e-5 in a TF32 gradient).  The
-//     synthesis path also has the grids of under 32 column tiles, where every
-//     form is a few launches of a few microseconds.
+//     synthesis path also has the grids of under 32 column tiles, in split BF16 as in
+//     the others: their test at Nt = 86 names its kernels.  Not for its time: the
+//     column form takes 0.70 to 0.78 of the inverse stages' time there up to 24
+//     channels (a forward with all lines, 4 x 2 x 20 x 20), 0.75 to 1.08 at 32.
 enum EpiKind { KIND_F32, KIND_COL, KIND_TC, KIND_MMA, KIND_SYNTH };
+
+// Tiles of 16 planes of the column epilogue so empty that the former kernel is faster
+// (forward with all lines, column form against it; C channels).  On the grids of
+// k_epi_mma: 64 x 64 x 4 x 32 134 : 126 at 20 channels, 154 : 131 at 24, 238 : 143 at 28;
+// 64 x 64 x 8 x 32 254 : 223 at 28; 64 x 64 x 20 x 32 422 : 387 at 28, and 420 : 439 with 24
+// planes.  On the others: 64 x 64 x 4 x 20 164 : 158 at 24, 261 : 192 at 28, and 281 : 278 with
+// 8 planes; grids of few tiles gain in any case (16 x 16 x 4 x 20 51 : 60 at 28).
+static bool col_thin(const Dims& d, int C, bool fused, int64_t tiles) {
+  if (fused) return d.Nz < 8 ? C > 20 : C > 24 && 4 * d.Nz < 3 * (16 * ((d.Nz + 15) / 16));
+  return d.Nz <= 4 && C > 24 && tiles >= 1024;
+}
+
 static EpiKind epilogue_kind(const Dims& d, int mode, int Cs, int Cl, int precision, bool region) {
   if (!is_tc(precision)) return KIND_F32;
   const bool fused = epilogue_mma_supported(d, mode, Cs, Cl, nullptr, 0);
@@ -387,11 +405,14 @@ static EpiKind epilogue_kind(const Dims& d, int mode, int Cs, int Cl, int precis
   const int C = std::max(Cs, Cl);
   const bool tc = is_split(precision) && epilogue_tc_supported(d, mode, Cs, Cl, nullptr, 0);
   if (tc && C > 24) return KIND_TC;
-  const bool tiny = d.B * d.Nx * d.Ny * ((d.Nz + 15) / 16) < 32;
-  if ((fused || (synth && !tiny)) &&
-      (precision == FNO_BF16X3 || (precision == FNO_BF16 && fused && mode != EPI_FWD)) &&
-      epilogue_col_supported(d, mode, Cs, Cl))
-    return KIND_COL;
+  const int64_t tiles = d.B * d.Nx * d.Ny * ((d.Nz + 15) / 16);
+  bool col = (fused || (synth && tiles >= 32)) && epilogue_col_supported(d, mode, Cs, Cl);
+  if (mode != EPI_SPECTRAL && col_thin(d, C, fused, tiles)) col = false;
+  if (precision == FNO_BF16) {
+    col = col && fused && mode != EPI_FWD;
+    if (mode == EPI_DX && (C > 24 || (d.Nz < 8 && C > 12))) col = false;
+  }
+  if (col && precision != FNO_TF32) return KIND_COL;
   return tc ? KIND_TC : fused ? KIND_MMA : synth ? KIND_SYNTH : KIND_F32;
 }
 
