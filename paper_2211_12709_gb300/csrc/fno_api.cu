@@ -452,18 +452,24 @@ static cudaError_t epilogue(const Dims& d, EpiArgs a, int precision, char* base,
   return launch_epilogue_f32(d, a, grid_used, s);
 }
 
-// Split BF16 beyond the two-CTA form of the dA pass (25..32 outputs or 32 inputs), on
-// the grids of k_epi_mma: the pass contracts dW_lin on the tensor cores in its wide
-// form, in place of the tensor-core dA epilogue, which evaluates A again (32
-// channels, 2 x 64^3 x 32: 2284 us and 20 more in the forward, against 4805).  Error of
-// dW_lin against 64 bits at 28 channels, 16 x 16 x 32 x 16: 3.3e-7 with that epilogue,
-// 2.8e-7 here.  In FP32, and on other grids, FP32 pair blocks form dW_lin: 2.3e-7
-// there (28 channels; this pass 2.6e-7), so they stay, though slower (64^3 x 16, 32
-// channels: 1692 us, against 579).
+// Where the dA pass of a tensor-core precision runs in its wide form (one CTA on an
+// SM), which contracts dW_lin on the tensor cores, beyond the two-CTA form (25..32
+// outputs or 32 inputs):
+//   In split BF16 on the grids of k_epi_mma, in place of the tensor-core dA epilogue,
+//     which evaluates A again (32 channels, 2 x 64^3 x 32: 2284 us and 20 more in the
+//     forward, against 4805).  Error of dW_lin against 64 bits at 28 channels, 16 x 16 x
+//     32 x 16: 3.3e-7 with that epilogue, 2.8e-7 here.
+//   On other grids, where the FP32 pair blocks sum each tile's 256 points in one
+//     chain (29..32 outputs with 32 inputs): dW_lin 3.1e-7 and db 3.2e-7 with them at 32
+//     channels, 16 x 16 x 32 x 20, 2.7e-7 and 1.9e-7 here (24 x 24 x 32 x 20: 167 us and 62).
+// Pair blocks with shorter chains are more exact than this pass (28 channels: 2.3e-7
+// against 2.8e-7 at Nt = 86) and stay; FNO_FP32 keeps FP32 products throughout (64^3 x
+// 16, 32 channels: 1692 us).
 static bool wide_da(const Dims& d, int precision) {
-  return precision == FNO_BF16X3 && !pointwise_da_mma_fits((int)d.Ci, (int)d.Co) &&
-         pointwise_da_mma_wide_fits((int)d.Ci, (int)d.Co) &&
-         epilogue_mma_supported(d, EPI_DA, (int)d.Co, (int)d.Ci, nullptr, 0);
+  const int Ci = (int)d.Ci, Co = (int)d.Co;
+  if (!is_tc(precision) || pointwise_da_mma_fits(Ci, Co) || !pointwise_da_mma_wide_fits(Ci, Co)) return false;
+  if (epilogue_mma_supported(d, EPI_DA, Co, Ci, nullptr, 0)) return precision == FNO_BF16X3;
+  return pointwise_da_pairs_one_chain(Ci, Co);
 }
 
 // Whether a training forward keeps GELU'(A) for the backward's dA pass.  The

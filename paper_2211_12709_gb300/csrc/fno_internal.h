@@ -166,6 +166,7 @@ int pointwise_max_grid(int Ci, int Co);  // the most rows launch_pointwise_bwd w
 // always where it fits two CTAs on an SM, in its one-CTA form where wide is set
 bool pointwise_da_mma_fits(int Ci, int Co);       // two CTAs on an SM
 bool pointwise_da_mma_wide_fits(int Ci, int Co);  // one
+bool pointwise_da_pairs_one_chain(int Ci, int Co);  // the CUDA-core form sums a tile in one chain
 cudaError_t launch_pointwise_bwd_saved(const float* x, const float* g, const float* dz, float* da,
                                        float* part, int max_rows, int64_t B, int64_t P, int Ci,
                                        int Co, bool wide, int* rows_out, cudaStream_t s);

@@ -38,9 +38,9 @@
 // The block backward after a training forward uses the same staging for its
 // dA pass: dA = dz GELU'(A) from the forward's saved GELU'(A), written out,
 // with the (dW_lin, db) partial sums.  Up to 31 inputs and 24 outputs, and up to 32
-// and 32 where its caller asks for it (split BF16), that contraction runs on the
-// tensor cores (k_da_mma, split TF32 products); wider layers take the FP32 pair
-// blocks of k_pw_bwd.
+// and 32 where its caller asks for it, that contraction runs on the tensor cores
+// (k_da_mma, split TF32 products); otherwise it takes the FP32 pair blocks of
+// k_pw_bwd.
 #include <algorithm>
 
 #include "fno_internal.h"
@@ -987,6 +987,7 @@ cudaError_t launch_pointwise_bwd(const float* x, const float* w, const float* bi
 // CTAs per SM still fit), shared-memory bytes
 bool pointwise_da_mma_fits(int Ci, int Co) { return Ci + 1 <= 16 * kDaMT && Co <= 8 * kDaNT; }
 bool pointwise_da_mma_wide_fits(int Ci, int Co) { return Ci <= 32 && Co <= 8 * kDaNTWide; }
+bool pointwise_da_pairs_one_chain(int Ci, int Co) { return pw_plan(Ci, Co, true).S == 1; }
 static void da_mma_plan(int Ci, int Co, int& nstage, size_t& smem) {
   const size_t stage = sizeof(float) * (size_t)(Ci + 1 + 2 * Co) * kPwLd;
   nstage = (2 * stage <= (size_t)(pointwise_da_mma_fits(Ci, Co) ? 110 : 226) * 1024) ? 2 : 1;

@@ -1,12 +1,13 @@
 """dW_lin and db of a training step beyond the two-CTA dA pass (25 to 32 outputs, 32 inputs and more).
 
 FP32, and the tensor-core precisions on grids that the tensor-core dA epilogue does
-not tile, form them in FP32: with one nonzero dA = 1 per output channel dW_lin is
-a value of x, all 24 bits of it.  (w = 0, w_lin = 0 and bias = 50 make A exactly
-50, where GELU' is exactly 1 in every form.)  Split BF16 on the other grids takes the
-wide tensor-core pass: its channel bounds, both counts of m-tiles, a partly
-filled tile of points and more than one batch entry against the FP64 oracle, with
-the bound of the block tests (1e-5).
+not tile (but at 32 -> 29..32), form them in FP32: with one nonzero dA = 1 per output
+channel dW_lin is a value of x, all 24 bits of it.  (w = 0, w_lin = 0 and bias = 50
+make A exactly 50, where GELU' is exactly 1 in every form.)  Split BF16 on the other
+grids, and the tensor-core precisions at 32 -> 29..32, take the wide tensor-core
+pass: its channel bounds, both counts of m-tiles, a partly filled tile of points and
+more than one batch entry against the FP64 oracle, with the bound of the block tests
+(1e-5).
 """
 import numpy as np
 import pytest
@@ -20,8 +21,8 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 EXACT = [("fp32", 28, 28, 16), ("fp32", 32, 32, 16), ("fp32", 33, 25, 10), ("fp32", 40, 28, 16), ("fp32", 47, 32, 7),
-         ("bf16x3", 28, 28, 20), ("bf16x3", 32, 32, 20), ("bf16x3", 40, 28, 16), ("tf32", 32, 32, 20),
-         ("bf16", 32, 32, 20)]
+         ("bf16x3", 28, 28, 20), ("bf16x3", 31, 32, 20), ("bf16x3", 40, 28, 16), ("tf32", 32, 28, 20),
+         ("bf16", 30, 32, 20)]
 
 
 @pytest.mark.parametrize("precision,ci,co,nt", EXACT, ids=["-".join(map(str, c)) for c in EXACT])
@@ -52,6 +53,8 @@ WIDE = [
     Dims(1, 32, 24, 4, 4, 12, 32, 2, 2, 4, 8),
     Dims(2, 9, 32, 3, 5, 16, 32, 1, 2, 4, 8),
     Dims(1, 1, 27, 3, 3, 8, 16, 1, 1, 4, 5),
+    Dims(1, 32, 32, 5, 4, 12, 20, 2, 1, 4, 6),
+    Dims(2, 32, 29, 3, 4, 10, 34, 1, 2, 3, 8),
 ]
 
 
