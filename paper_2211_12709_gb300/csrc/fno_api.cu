@@ -100,7 +100,6 @@ int sm_count() {
 // ---- validation and workspace layout ---------------------------------------
 static const int64_t kMaxChannels = 64;
 static const int64_t kMaxModesT = 16;
-static const size_t kMaxSmem = 227 * 1024;
 
 static int to_dims(const fno_dims* dd, Dims* d) {
   if (!dd) return fail(FNO_ERR_INVALID_ARG, "dims is NULL");

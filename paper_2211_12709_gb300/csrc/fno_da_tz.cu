@@ -648,8 +648,7 @@ bool da_tz_supported(const Dims& d, char* why, size_t nwhy) {
 
 template <bool SPLIT, bool TF, int MZ>
 static cudaError_t launch_da_tz_t(const DaTz& k, size_t smem, int grid, const char* name, cudaStream_t s) {
-  cudaError_t e =
-      cudaFuncSetAttribute(k_da_tz<SPLIT, TF, MZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)k_da_tz<SPLIT, TF, MZ>, smem);
   if (e != cudaSuccess) return e;
   FNO_LAUNCH(name, (k_da_tz<SPLIT, TF, MZ>), grid, kDtThreads, smem, s, k);
   return cudaSuccess;

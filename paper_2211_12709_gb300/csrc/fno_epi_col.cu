@@ -427,7 +427,7 @@ static cudaError_t launch_col_t(EpiCol k, const char* name, cudaStream_t s) {
                       sizeof(ulonglong2) * (size_t)k.NPAIR * CM + sizeof(float2) * (size_t)((k.NPAIR + 1) & ~1) +
                       sizeof(float2) * (size_t)k.a.Cs * k.Jz * k.Jt;
   const void* kern = (const void*)k_epi_col<MODE, CM, NP, H, CH, NW, MINB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)

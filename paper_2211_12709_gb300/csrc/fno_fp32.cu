@@ -32,11 +32,6 @@ static int persistent_grid(const void* kern, int threads, size_t smem, int64_t w
   return (int)g;
 }
 
-static cudaError_t allow_smem(const void* kern, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 // ---------------------------------------------------------------------------
 // Basis tables: exp(sign * 2 pi i * (k n mod N) / N), evaluated in FP64 with
 // sincospi on the exactly reduced residue, optionally scaled by c(kt)/Ng.
@@ -580,7 +575,7 @@ static int tzf_warps(const Dims& d, TzfRows rows) {
 static int tzf_warps_per_sm(const Dims& d, TzfRows rows) {
   const int W = tzf_warps(d, rows);
   const size_t smem = tzf_smem(d, rows, W);
-  if (smem > 227 * 1024) return 0;
+  if (smem > kMaxSmem) return 0;
   return W * (int)std::min<size_t>(3, 228 * 1024 / (smem + 1024));
 }
 
@@ -1001,10 +996,8 @@ template <int BC>
 static cudaError_t launch_mix_bc(const Dims& d, const float2* xh, const float2* w, float2* yh,
                                  cudaStream_t s) {
   const size_t smem = sizeof(float2) * (size_t)BC * (size_t)d.Ci * kMixJ;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_mix_f32<BC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = allow_smem((const void*)k_mix_f32<BC>, smem);
+  if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)((d.Mk + kMixJ - 1) / kMixJ);
   int groups = mix_groups(d.Co, grid);
   if (mix_widen(BC * d.Ci, groups, grid)) groups = kMixMin;

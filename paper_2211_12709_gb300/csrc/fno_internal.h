@@ -203,6 +203,17 @@ cudaError_t launch_da_tz(const float* x, const float* g, const float* dz, float*
 
 #ifdef __CUDACC__
 // Launch with the profiling hooks; returns the launch error from the caller.
+// Raises a kernel's dynamic shared-memory limit for a launch with smem bytes, to
+// the most that an SM gives one CTA: always the same value, so that a thread never
+// lowers the limit between another one's call of this and its launch.  (No kernel
+// here has static shared memory beside a dynamic window of that size.)
+constexpr size_t kMaxSmem = 227 * 1024;
+inline cudaError_t allow_smem(const void* kern, size_t smem) {
+  if (smem <= 48 * 1024) return cudaSuccess;
+  if (smem > kMaxSmem) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
 #define FNO_LAUNCH(name, kern, grid, block, smem, stream, ...)   \
   do {                                                           \
     prof_before(name, stream);                                   \

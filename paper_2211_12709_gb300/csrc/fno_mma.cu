@@ -851,7 +851,7 @@ template <int MODE, bool SPLIT, bool TF>
 static cudaError_t launch_mma_t(const EpiM& k, int* grid_used, cudaStream_t s) {
   const void* kern = (const void*)k_epi_mma<MODE, SPLIT, TF>;
   const size_t smem = k.off[R_END];
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) != cudaSuccess ||
@@ -1163,7 +1163,7 @@ bool line_mma_supported(int nin, int nout) {
 template <bool SPLIT, bool KOUTER, bool TF>
 static cudaError_t launch_line_t(const LineM& L, size_t smem, const char* name, cudaStream_t s) {
   const void* kern = (const void*)k_line_mma<SPLIT, KOUTER, TF>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem) != cudaSuccess || per_sm < 1)
@@ -1348,7 +1348,7 @@ bool synth_t_supported(int Nt, int Jt) { return Nt >= 1 && Nt <= 8 * kSynthNTMax
 
 template <bool SPLIT, bool TF>
 static cudaError_t launch_synth_k(const SynthT& k, size_t smem, const char* name, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_synth_t<SPLIT, TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)k_synth_t<SPLIT, TF>, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_synth_t<SPLIT, TF>, 256, smem) != cudaSuccess ||
@@ -1775,8 +1775,7 @@ bool fwd_tz_mma_supported(const Dims& d, char* why, size_t nwhy) {
 
 template <int MZ, int KTR, bool SPLIT, bool TF>
 static cudaError_t launch_tz_t(const TzM& k, size_t smem, const char* name, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_fwd_tz_mma<MZ, KTR, SPLIT, TF>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)k_fwd_tz_mma<MZ, KTR, SPLIT, TF>, smem);
   if (e != cudaSuccess) return e;
   const int grid =
       (int)std::max<long long>(1, std::min<long long>((long long)tz_ctas(MZ) * sm_count(), k.nunits));

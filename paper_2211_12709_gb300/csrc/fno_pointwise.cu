@@ -775,11 +775,6 @@ static const void* pw_bwd_kernel(int KB) {
   }
 }
 
-static void allow_smem(const void* kern, size_t smem) {
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 size_t pointwise_smem_bytes(int Ci, int Co, bool saved_grad) {
   return pw_plan(Ci, Co, saved_grad).smem;
 }

@@ -833,7 +833,7 @@ size_t epilogue_tc_table_bytes(const Dims& d) {
 template <int MODE, bool SPLIT, bool X3, bool TF, int CH>
 static cudaError_t launch_tc_c(const EpiTc& k, cudaStream_t s, const char* name) {
   const void* kern = (const void*)k_epi_tc<MODE, SPLIT, X3, TF, CH>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+  cudaError_t e = allow_smem(kern, k.smem);
   if (e != cudaSuccess) return e;
   long long g = sm_count();
   if (g > k.ngroups) g = k.ngroups;

@@ -249,7 +249,7 @@ template <int MZ, int KT, bool SPLIT, bool TF>
 static cudaError_t launch_tzr_t(const TzR& k, const char* name, cudaStream_t s) {
   const size_t smem = 16 * 32 * ((size_t)MZ * k.KZ * 4 + (KT <= 2 ? 0 : 2 * KT));
   const void* kern = (const void*)k_fwd_tz_reg<MZ, KT, SPLIT, TF>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTzrWarps, smem) != cudaSuccess || per_sm < 1)
