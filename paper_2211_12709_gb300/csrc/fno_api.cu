@@ -440,7 +440,7 @@ static cudaError_t epilogue(const Dims& d, EpiArgs a, int precision, char* base,
                                  a.It == tables_at(base, L).Its, s);
     }
     case KIND_TC:
-      return launch_epilogue_tc(d, a, true, tf32, base + L.tc_tab, err, s);
+      return launch_epilogue_tc(d, a, tf32, base + L.tc_tab, err, s);
     case KIND_MMA:
       return launch_epilogue_mma(d, a, split, tf32, base + L.mma_tab, err, grid_used, s);
     case KIND_SYNTH:

@@ -463,7 +463,7 @@ static cudaError_t launch_col_c(const EpiCol& k, bool narrow, bool fine, const c
       if (fine) return launch_col_t<MODE, 24, NP, 2, C4, NW, MINB>(k, name, s);
       return launch_col_t<MODE, 24, NP, 2, C1, NW, MINB>(k, name, s);
     }
-    return launch_col_t<MODE, 32, NP, 2, C4, 4, 2>(k, name, s);
+    if constexpr (NP > 1) return launch_col_t<MODE, 32, NP, 2, C4, 4, 2>(k, name, s);
   } else {
     if (k.a.Cl <= 8) return launch_col_t<MODE, 8, NP, 1, C1, 4, 5>(k, name, s);
     if (k.a.Cl <= 20) {
@@ -474,15 +474,17 @@ static cudaError_t launch_col_c(const EpiCol& k, bool narrow, bool fine, const c
       if (fine) return launch_col_t<MODE, 24, NP, 1, C4, 4, 4>(k, name, s);
       return launch_col_t<MODE, 24, NP, 1, C1, 4, 4>(k, name, s);
     }
-    return launch_col_t<MODE, 32, NP, 1, C4, 8, 2>(k, name, s);
+    if constexpr (NP > 1) return launch_col_t<MODE, 32, NP, 1, C4, 8, 2>(k, name, s);
   }
+  return cudaErrorInvalidValue;  // not reached: plain BF16 has at most 24 inputs here
 }
 
 template <int NP>
 static cudaError_t launch_col_m(const EpiCol& k, bool narrow, bool fine, const char* name, cudaStream_t s) {
   if (k.a.mode == EPI_SPECTRAL) return launch_col_c<EPI_SPECTRAL, NP>(k, narrow, fine, name, s);
   if (k.a.mode == EPI_DX) return launch_col_c<EPI_DX, NP>(k, narrow, fine, name, s);
-  return launch_col_c<EPI_FWD, NP>(k, narrow, fine, name, s);
+  if constexpr (NP > 1) return launch_col_c<EPI_FWD, NP>(k, narrow, fine, name, s);
+  return cudaErrorInvalidValue;  // not reached: plain BF16 runs its forward on k_epi_mma
 }
 
 cudaError_t launch_epilogue_col(const Dims& d, const EpiArgs& a, bool split, bool exact, bool lin_round,
@@ -508,8 +510,8 @@ cudaError_t launch_epilogue_col(const Dims& d, const EpiArgs& a, bool split, boo
   k.nunits = (unsigned)(d.B * k.NxNy * ct.NZ);
   static const char* const names[4][2] = {{"fno_epi_spectral_cmma_bf16", "fno_epi_spectral_cmma_bf16x3"},
                                           {"fno_epi_dx_cmma_bf16", "fno_epi_dx_cmma_bf16x3"},
-                                          {"fno_epi_fwd_cmma_bf16", "fno_epi_fwd_cmma_bf16x3"},
-                                          {"fno_epi_fwd_train_cmma_bf16", "fno_epi_fwd_train_cmma_bf16x3"}};
+                                          {"", "fno_epi_fwd_cmma_bf16x3"},
+                                          {"", "fno_epi_fwd_train_cmma_bf16x3"}};
   const char* name = names[a.mode == EPI_SPECTRAL ? 0 : a.mode == EPI_DX ? 1 : a.gp ? 3 : 2][split ? 1 : 0];
   const bool narrow = ct.H == 2;
   if (!split) return launch_col_m<1>(k, narrow, fine, name, s);

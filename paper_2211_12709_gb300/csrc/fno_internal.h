@@ -124,7 +124,7 @@ cudaError_t launch_epilogue_col(const Dims& d, const EpiArgs& a, bool split, boo
 // scratch of epilogue_tc_table_bytes(d) for the z basis images.
 bool epilogue_tc_supported(const Dims& d, int mode, int Cs, int Cl, char* why, size_t nwhy);
 size_t epilogue_tc_table_bytes(const Dims& d);
-cudaError_t launch_epilogue_tc(const Dims& d, const EpiArgs& a, bool split, bool tf32, void* table, int* err,
+cudaError_t launch_epilogue_tc(const Dims& d, const EpiArgs& a, bool tf32, void* table, int* err,
                                cudaStream_t s);
 
 // One complex DFT axis on mma.sync (fno_mma.cu), BF16 (one product), split

@@ -880,7 +880,10 @@ static cudaError_t launch_mma_t(const EpiM& k, int* grid_used, cudaStream_t s) {
 template <int MODE>
 static cudaError_t launch_mma_m(const EpiM& k, bool split, bool tf32, int* g, cudaStream_t s) {
   if (tf32) return launch_mma_t<MODE, true, true>(k, g, s);
-  return split ? launch_mma_t<MODE, true, false>(k, g, s) : launch_mma_t<MODE, false, false>(k, g, s);
+  // the column epilogue takes the spectral form of the BF16 precisions on every grid
+  // of this kernel
+  if constexpr (MODE == EPI_SPECTRAL) return cudaErrorInvalidValue;
+  else return split ? launch_mma_t<MODE, true, false>(k, g, s) : launch_mma_t<MODE, false, false>(k, g, s);
 }
 
 // Tiled tensor map of an FP32 array, encoded through the driver entry point

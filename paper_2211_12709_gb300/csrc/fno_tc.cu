@@ -850,20 +850,18 @@ static cudaError_t launch_tc_t(const EpiTc& k, cudaStream_t s, const char* name)
 }
 
 template <int MODE>
-static cudaError_t launch_tc_m(const EpiTc& k, bool split, bool tf32, cudaStream_t s) {
-  static const char* names[3][4] = {
-      {"fno_epi_spectral_tc_bf16", "fno_epi_fwd_tc_bf16", "", "fno_epi_dx_tc_bf16"},
+static cudaError_t launch_tc_m(const EpiTc& k, bool tf32, cudaStream_t s) {
+  static const char* names[2][4] = {
       {"fno_epi_spectral_tc_bf16x3", "fno_epi_fwd_tc_bf16x3", "", "fno_epi_dx_tc_bf16x3"},
       {"fno_epi_spectral_tc_tf32", "fno_epi_fwd_tc_tf32", "", "fno_epi_dx_tc_tf32"}};
-  static const char* train_names[3] = {"fno_epi_fwd_train_tc_bf16", "fno_epi_fwd_train_tc_bf16x3",
-                                       "fno_epi_fwd_train_tc_tf32"};
-  const int pv = tf32 ? 2 : (split ? 1 : 0);
+  static const char* train_names[2] = {"fno_epi_fwd_train_tc_bf16x3", "fno_epi_fwd_train_tc_tf32"};
+  const int pv = tf32 ? 1 : 0;
   const char* name = (MODE == EPI_FWD && k.a.gp) ? train_names[pv] : names[pv][MODE];
   if (tf32) return launch_tc_t<MODE, true, false, true>(k, s, name);
-  return split ? launch_tc_t<MODE, true, true, false>(k, s, name) : launch_tc_t<MODE, false, false, false>(k, s, name);
+  return launch_tc_t<MODE, true, true, false>(k, s, name);
 }
 
-cudaError_t launch_epilogue_tc(const Dims& d, const EpiArgs& a, bool split, bool tf32, void* table, int* err,
+cudaError_t launch_epilogue_tc(const Dims& d, const EpiArgs& a, bool tf32, void* table, int* err,
                                cudaStream_t s) {
   EpiTc k{};
   if (!tc_plan(d, a.mode, a.Cs, a.Cl, k, nullptr, 0)) return cudaErrorInvalidValue;
@@ -886,9 +884,9 @@ cudaError_t launch_epilogue_tc(const Dims& d, const EpiArgs& a, bool split, bool
                k.KZ1, tf32 ? 1 : 0, ngz, static_cast<uint16_t*>(table));
   }
   switch (a.mode) {
-    case EPI_SPECTRAL: return launch_tc_m<EPI_SPECTRAL>(k, split, tf32, s);
-    case EPI_FWD: return launch_tc_m<EPI_FWD>(k, split, tf32, s);
-    default: return launch_tc_m<EPI_DX>(k, split, tf32, s);
+    case EPI_SPECTRAL: return launch_tc_m<EPI_SPECTRAL>(k, tf32, s);
+    case EPI_FWD: return launch_tc_m<EPI_FWD>(k, tf32, s);
+    default: return launch_tc_m<EPI_DX>(k, tf32, s);
   }
 }
 
