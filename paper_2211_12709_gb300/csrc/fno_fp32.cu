@@ -777,7 +777,7 @@ cudaError_t launch_line_f32(const float2* in, float2* out, int64_t outer, int ni
     cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     const int grid = persistent_grid(k, 256, smem, outer * t2);
-    FNO_LAUNCH("fno_line_f32", k_line_pair_f32<4>, grid, dim3(32, 8), smem, s, in, out,
+    FNO_LAUNCH("fno_line_pair_f32", k_line_pair_f32<4>, grid, dim3(32, 8), smem, s, in, out,
                (long long)outer, nin, nout, (long long)inner, tab);
     return cudaSuccess;
   }
