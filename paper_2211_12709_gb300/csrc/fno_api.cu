@@ -451,23 +451,23 @@ static cudaError_t epilogue(const Dims& d, EpiArgs a, int precision, char* base,
   return launch_epilogue_f32(d, a, grid_used, s);
 }
 
-// Where the dA pass of a tensor-core precision runs in its wide form (one CTA on an
-// SM), which contracts dW_lin on the tensor cores, beyond the two-CTA form (25..32
-// outputs or 32 inputs):
+// Where the dA pass runs in its wide form (one CTA on an SM), which contracts dW_lin on
+// the tensor cores in split TF32, beyond the two-CTA form (25..32 outputs or 32
+// inputs):
 //   In split BF16 on the grids of k_epi_mma, in place of the tensor-core dA epilogue,
 //     which evaluates A again (32 channels, 2 x 64^3 x 32: 2284 us and 20 more in the
 //     forward, against 4805).  Error of dW_lin against 64 bits at 28 channels, 16 x 16 x
 //     32 x 16: 3.3e-7 with that epilogue, 2.8e-7 here.
-//   On other grids, where the FP32 pair blocks sum each tile's 256 points in one
-//     chain (29..32 outputs with 32 inputs): dW_lin 3.1e-7 and db 3.2e-7 with them at 32
-//     channels, 16 x 16 x 32 x 20, 2.7e-7 and 1.9e-7 here (24 x 24 x 32 x 20: 167 us and 62).
-// Pair blocks with shorter chains are more exact than this pass (28 channels: 2.3e-7
-// against 2.8e-7 at Nt = 86) and stay; FNO_FP32 keeps FP32 products throughout (64^3 x
-// 16, 32 channels: 1692 us).
+//   Otherwise where the FP32 pair blocks sum each tile's 256 points in one chain
+//     (29..32 outputs with 32 inputs) and are the less exact: at 32 channels, 16 x 16 x 32
+//     x 16 in FP32, dW_lin 3.0e-7 and db 3.2e-7 with them, 2.6e-7 and 1.7e-7 here (split
+//     BF16 at Nt = 20 3.1e-7 and 3.2e-7, 2.7e-7 and 1.9e-7); 64^3 x 16 1692 us, 579 here.
+// Pair blocks with shorter chains are more exact than this pass (28 channels, FP32:
+// 2.3e-7 against 2.6e-7) and stay.
 static bool wide_da(const Dims& d, int precision) {
   const int Ci = (int)d.Ci, Co = (int)d.Co;
-  if (!is_tc(precision) || pointwise_da_mma_fits(Ci, Co) || !pointwise_da_mma_wide_fits(Ci, Co)) return false;
-  if (epilogue_mma_supported(d, EPI_DA, Co, Ci, nullptr, 0)) return precision == FNO_BF16X3;
+  if (pointwise_da_mma_fits(Ci, Co) || !pointwise_da_mma_wide_fits(Ci, Co)) return false;
+  if (is_tc(precision) && epilogue_mma_supported(d, EPI_DA, Co, Ci, nullptr, 0)) return precision == FNO_BF16X3;
   return pointwise_da_pairs_one_chain(Ci, Co);
 }
 

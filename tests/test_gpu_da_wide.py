@@ -1,11 +1,11 @@
 """dW_lin and db of a training step beyond the two-CTA dA pass (25 to 32 outputs, 32 inputs and more).
 
 FP32, and the tensor-core precisions on grids that the tensor-core dA epilogue does
-not tile (but at 32 -> 29..32), form them in FP32: with one nonzero dA = 1 per output
+not tile, form them in FP32 but at 32 -> 29..32: with one nonzero dA = 1 per output
 channel dW_lin is a value of x, all 24 bits of it.  (w = 0, w_lin = 0 and bias = 50
 make A exactly 50, where GELU' is exactly 1 in every form.)  Split BF16 on the other
-grids, and the tensor-core precisions at 32 -> 29..32, take the wide tensor-core
-pass: its channel bounds, both counts of m-tiles, a partly filled tile of points and
+grids, and every precision at 32 -> 29..32, take the wide tensor-core pass, whose
+error there is the smaller one: its channel bounds, both counts of m-tiles, a partly filled tile of points and
 more than one batch entry against the FP64 oracle, with the bound of the block tests
 (1e-5).
 """
@@ -20,7 +20,7 @@ torch = pytest.importorskip("torch")
 
 pytestmark = pytest.mark.gpu
 
-EXACT = [("fp32", 28, 28, 16), ("fp32", 32, 32, 16), ("fp32", 33, 25, 10), ("fp32", 40, 28, 16), ("fp32", 47, 32, 7),
+EXACT = [("fp32", 28, 28, 16), ("fp32", 32, 28, 16), ("fp32", 33, 25, 10), ("fp32", 40, 28, 16), ("fp32", 47, 32, 7),
          ("bf16x3", 28, 28, 20), ("bf16x3", 31, 32, 20), ("bf16x3", 40, 28, 16), ("tf32", 32, 28, 20),
          ("bf16", 30, 32, 20)]
 
@@ -63,8 +63,12 @@ def relerr(a, b):
     return float(np.linalg.norm((a - b).ravel()) / np.linalg.norm(np.asarray(b).ravel()))
 
 
-@pytest.mark.parametrize("d", WIDE, ids=[f"{d.B}x{d.Ci}-{d.Co}x{d.Nz}x{d.Nt}" for d in WIDE])
-def test_wide_tensor_core_pass_matches_the_oracle(d):
+CHAIN = [("fp32", d) for d in (Dims(1, 32, 32, 4, 5, 16, 16, 2, 2, 4, 6), Dims(2, 32, 29, 3, 4, 9, 7, 1, 2, 3, 4))]
+RUNS = [("bf16x3", d) for d in WIDE] + CHAIN
+
+
+@pytest.mark.parametrize("precision,d", RUNS, ids=[f"{p}-{d.B}x{d.Ci}-{d.Co}x{d.Nz}x{d.Nt}" for p, d in RUNS])
+def test_wide_tensor_core_pass_matches_the_oracle(precision, d):
     from paper_2211_12709_gb300 import _lib, ops
     modes = (d.mx, d.my, d.mz, d.mt)
     x = inputs.normal((d.B, d.Ci) + d.grid, 811)
@@ -72,10 +76,10 @@ def test_wide_tensor_core_pass_matches_the_oracle(d):
     wl, b = inputs.linear_params(d.Ci, d.Co, 813)
     dz = inputs.normal((d.B, d.Co) + d.grid, 814)
     X, W, WL, Bb, DZ = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (x, w, wl, b, dz))
-    ws = ops.workspace(ops.dims_of(X, d.Co, modes), "bf16x3", ops.OP_BLOCK_TRAIN, X.device)
+    ws = ops.workspace(ops.dims_of(X, d.Co, modes), precision, ops.OP_BLOCK_TRAIN, X.device)
     _lib.fno_profile_start()
-    z = ops.block_fwd(X, W, WL, Bb, modes, "bf16x3", ws=ws, train=True)
-    got = ops.block_bwd(X, W, WL, Bb, DZ, modes, "bf16x3", ws=ws, saved=True)
+    z = ops.block_fwd(X, W, WL, Bb, modes, precision, ws=ws, train=True)
+    got = ops.block_bwd(X, W, WL, Bb, DZ, modes, precision, ws=ws, saved=True)
     torch.cuda.synchronize()
     names = _lib.fno_profile_stop()
     assert "fno_da_saved" in names, sorted(names)
