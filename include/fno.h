@@ -59,7 +59,9 @@ typedef struct fno_dims {
 } fno_dims;
 
 /* Arithmetic of the contractions (accumulation is always FP32):
- *   FNO_FP32    FP32 on the CUDA cores (the plain form)
+ *   FNO_FP32    FP32 on the CUDA cores (the plain form; a training step's dW_lin
+ *               and db up to 31 inputs and 24 outputs, and at 32 -> 29..32, as split
+ *               TF32 with FP32-size errors)
  *   FNO_TF32    TF32 numerics: every tensor-core operand rounded to TF32
  *               (nearest), exact products; a TF32 value is exact as BF16
  *               hi + lo, so it runs as split products on the BF16 tensor
@@ -67,19 +69,21 @@ typedef struct fno_dims {
  *   FNO_BF16    BF16 tensor-core products (one product)
  *   FNO_BF16X3  split BF16 on the tensor cores: hi + lo with three products
  *               in the DFT stages, three-way splits with six products in the
- *               line stages; the 1x1 in FP32 (above 24 channels as 3xTF32 on
- *               tcgen05: big + small parts, three products, FP32-like)
+ *               line stages; the 1x1 in FP32 (as 3xTF32 on tcgen05 above 24
+ *               channels, big + small parts, three products, FP32-like, and as
+ *               three-way splits on mma.sync)
  * The tensor-core precisions need Nt even and at most 128, Nz * Nt a multiple
  * of 4, mt <= 8 and 2 mz <= 64 (FNO_ERR_UNSUPPORTED otherwise).  The inverse z, t +
  * epilogue stage of FNO_BF16X3 is one kernel on warp-level mma.sync and packed
  * FP32 (the column epilogue) with up to 32 channels, and on tcgen05 (TMEM
  * accumulators) with more than 24 channels at Nt = 16 or 32, Nz a multiple of
  * 512 / Nt, 2 mz <= 24.  FNO_TF32 runs on tcgen05 there with any channel count;
- * FNO_BF16 on warp-level mma.sync (dX and the spectral form on the column
- * epilogue); the dA pass of fno_block_bwd on mma.sync.  For other Nt (the paper's
- * 84 and 86), with mt <= 8, up to 32 channels and the inverse z stage within the
- * tensor-core line tiling, FNO_TF32 and FNO_BF16 (and grids of fewer than 32
- * tiles of 16 planes) take a synthesis path: the inverse z stage and the inverse
+ * FNO_BF16 on warp-level mma.sync (dX up to 24 channels and the spectral form on
+ * the column epilogue), and FNO_BF16X3 too where the column epilogue's tiles of
+ * 16 planes would be mostly empty; the dA pass of fno_block_bwd on mma.sync.  For
+ * other Nt (the paper's 84 and 86), with mt <= 8, up to 32 channels and the inverse
+ * z stage within the tensor-core line tiling, FNO_TF32 and FNO_BF16 (and grids of
+ * fewer than 32 tiles of 16 planes) take a synthesis path: the inverse z stage and the inverse
  * t stage to real points on mma.sync, the second written straight into the
  * output, then the 1x1, bias and GELU in FP32 in place (a workspace region of B *
  * max(C_in, C_out) * Nx * Ny * Nz * mt complex values holds the z stage and is

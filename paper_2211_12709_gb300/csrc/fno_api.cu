@@ -368,9 +368,9 @@ static cudaError_t synth_epilogue(const Dims& d, const EpiArgs& a, int precision
 //     1005 at 16, 1280 : 1437 at 24; against the synthesis path, Nt = 86: 1047 :
 //     1860 at 8 channels, 502 : 1370 at 4, 5531 : 7881 at 32.
 //     Not where many of the planes of its tiles of 16 do not exist (col_thin), nor
-//     plain BF16 dX above 24 channels, where k_epi_mma is as fast or faster (dX alone,
-//     column form against it: 64^3 x 32 channels 246 : 220 at Nt = 16, 24 channels 73 : 70
-//     at 32 x 32 x 64 x 16; 64 x 64 x 8 x 16 at 28 channels 99 : 72).
+//     plain BF16 dX above 24 channels, where k_epi_mma is the faster mostly (dX alone,
+//     column form against it, 32 x 32 x 64 x 16: 59 : 67 at 20 channels, 73 : 70 at 24, 112 :
+//     80 at 28, 123 : 110 at 32; 64 x 64 x 8 x 16 99 : 72 at 28).
 //   tcgen05 (k_epi_tc): beyond 24 channels, where its 32-wide products are full
 //     and the FP32 1x1 of the column form no longer is cheaper (Nt = 32, 32
 //     channels: 1502 : 1774; 24 channels: 1437 : 1280, at Nt = 16 807 : 721); and
@@ -380,9 +380,9 @@ static cudaError_t synth_epilogue(const Dims& d, const EpiArgs& a, int precision
 //     rounded to 11 or 8 bits later, and a sum that differs in its last bit
 //     turns some of those roundings (rel 5e-5 in a TF32 gradient).  The
 //     synthesis path also has the grids of under 32 column tiles, in split BF16 as in
-//     the others: their test at Nt = 86 names its kernels.  Not for its time: the
-//     column form takes 0.70 to 0.78 of the inverse stages' time there up to 24
-//     channels (a forward with all lines, 4 x 2 x 20 x 20), 0.75 to 1.08 at 32.
+//     the others: their test at Nt = 86 names its kernels.  Not for its time: on 4 to 32
+//     tiles the column form takes 0.68 to 0.97 of the time of a forward's lines and
+//     epilogue up to 24 channels (median 0.75), 0.74 to 1.09 at 32.
 enum EpiKind { KIND_F32, KIND_COL, KIND_TC, KIND_MMA, KIND_SYNTH };
 
 // Tiles of 16 planes of the column epilogue so empty that the former kernel is faster

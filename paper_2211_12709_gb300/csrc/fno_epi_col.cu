@@ -1,8 +1,8 @@
 // fno_epi_col.cu -- the last stage of the inverse transform of Alg. 2 (inverse
 // z, then inverse t; Sec. IV-C runs the inverse as the adjoint of the forward
 // DFT) fused with the block's pointwise 1x1 channel linear, bias and GELU, for
-// split BF16 and plain BF16 and any even Nt up to 128 (modes EPI_FWD, EPI_DX and
-// EPI_SPECTRAL).
+// split BF16 and any even Nt up to 128 (modes EPI_FWD, EPI_DX and EPI_SPECTRAL), and
+// for plain BF16 in the last two.
 //
 // Work unit: 16 z-planes of one (b, x, y) column, every channel, by a CTA of
 // four to eight warps.
@@ -36,7 +36,8 @@
 // A packed FMA takes 2.3 cycles a scheduler, an mma.sync of this shape 8 (tf32
 // m16n8k8 as well, for half the products).  At Nt = 84 and 86 a unit has twelve
 // items, and what decides is L1: rows of 336 or 344 bytes share sectors and lines
-// between items.  Forward + dX at 262 x 118 x 64 x 86 and forward at 130^3 x 84:
+// between items.  Training forward + dX at 262 x 118 x 64 x 86 and training forward
+// (with GELU'(A)) at 130^3 x 84:
 // two CTAs of six warps 18.4 and 12.4 ms, two of four 20.7 and 13.8, three of
 // four 22.1 and 17.8, one of eight 24.6 and 16.5 (synthesis path 34.0 and 20.7;
 // HBM asks for 10.4 and 6.6).  A form that took 14 ms for the forward there took 9
@@ -441,7 +442,7 @@ static cudaError_t launch_col_t(EpiCol k, const char* name, cudaStream_t s) {
 // error at Nt = 84 1.29e-7 against 1.47e-7 in one, in the same time).  With two parts
 // one chain of up to 24 channels is more exact than the tcgen05 form's 3xTF32 was
 // (z 1.6e-7 against 2.4e-7 at 20 channels); four chains are for what replaces the
-// six-product 1x1 of k_epi_mma (fine): z 1.61e-7 with one and 1.16e-7 with four
+// six-product 1x1 of k_epi_mma (fine): z 1.62e-7 with one and 1.16e-7 with four
 // chains, 1.18e-7 in k_epi_mma, at 32 channels and Nt = 16, in the same time (32
 // channels: 488 us a dX either way at 64^3 x 16).  At 20 channels and Nt = 32 they
 // cost 4 to 7 %.

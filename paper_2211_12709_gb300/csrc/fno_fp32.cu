@@ -811,7 +811,7 @@ cudaError_t launch_line_f32(const float2* in, float2* out, int64_t outer, int ni
 // HBM bounds it (W, and dW in the adjoint).  With 16 fixed groups (20 channels:
 // two rounds, the second a quarter full) and 4 or 8 weights in flight the
 // forward and its adjoint took 59 and 57 us at 24576 modes, B = 2, width 20 (W 79
-// MB), here 27 and 42; 72 and 107, here 53 and 94 at 73728 modes, B = 1; 263 and
+// MB), here 27 and 42; 72 and 107, here 51 and 87 at 73728 modes, B = 1; 263 and
 // 361, here 207 and 354 at 110592 modes, B = 2, width 32.  20 weights in flight
 // measured slower (registers), 5 about as fast.  One group and no more for a single
 // channel (20 -> 1 forward, 1 -> 20 adjoint, 24576 modes, B = 16) took 304 and 360 us,
